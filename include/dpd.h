@@ -223,9 +223,10 @@ DPD_API int64_t dpd_num_particles(const dpd_ctx *ctx);
 
 /* ------------------------------------------------------- instrumentation */
 #define DPD_NUM_STAGES 5       /* integrate+count, scan, key pass, reorder, force */
-#define DPD_KERNELS_PER_STEP 7 /* kernel launches per step of one force band with the full
-                                 * stencil (the scan takes three); the half stencil has no
-                                 * key pass: one fewer */
+#define DPD_KERNELS_PER_STEP 6 /* kernel launches per step of one force band with the full
+                                 * stencil (the scan takes two; one below 4096 cell slices,
+                                 * three above 2048 x 4096); the half stencil has no key
+                                 * pass: one fewer */
 
 /* Advance nsteps steps like dpd_step, launching each step's kernels directly
  * (no graph) with CUDA events recorded on the context's stream between the

@@ -8,7 +8,8 @@
 //                     (Sec. 3.2); with the full stencil the previous step's
 //                     force kernel can do this instead (fused);
 //   2. scan           exclusive scan of the cell counts into cell starts
-//                     (three passes: tile sums, scan of the tile sums, apply);
+//                     (one pass for one tile, two up to 2048 tiles, else three:
+//                     tile sums, scan of the tile sums, apply);
 //   3. bin_keys       full stencil: record each slot's old index at its
 //                     arrival position;
 //   4. bin_scatter    move position and velocity to the new slot: full
@@ -141,7 +142,10 @@ __global__ void __launch_bounds__(1024) k_scan_bsum(int *__restrict__ bsum, int 
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_apply(Packed P, bool advance) {
+// sum_tiles: bsum holds the tiles' sums, and each block adds up those before
+// its own; otherwise it holds their exclusive scan.
+__global__ void __launch_bounds__(kScanThreads)
+    k_scan_apply(Packed P, bool advance, bool sum_tiles) {
   int4 *c4 = reinterpret_cast<int4 *>(P.count) + (size_t)blockIdx.x * (kScanTile / 4) +
              threadIdx.x * (kScanItems / 4);
   int4 *s4 = reinterpret_cast<int4 *>(P.start) + (size_t)blockIdx.x * (kScanTile / 4) +
@@ -160,7 +164,15 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(Packed P, bool adva
 #pragma unroll
   for (int k = 0; k < kScanItems; ++k) s += v[k];
   int total;
-  int run = block_excl_scan<kScanThreads>(s, &total) + P.bsum[blockIdx.x];
+  int run = block_excl_scan<kScanThreads>(s, &total);
+  if (sum_tiles) {
+    int before = 0;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += kScanThreads) before += P.bsum[k];
+    block_excl_scan<kScanThreads>(before, &total);
+    run += total;
+  } else {
+    run += P.bsum[blockIdx.x];
+  }
 #pragma unroll
   for (int k = 0; k < kScanItems / 4; ++k) {
     int4 o;
@@ -559,6 +571,21 @@ cudaError_t launch_load(const Packed &P, int slot0, int n, const float *pos3, co
   return cudaGetLastError();
 }
 
+// Scan of the cell counts.  One tile needs no sums of others.  Up to
+// kScanSumTiles tiles each block of the last pass adds up the sums before its
+// own (at most 8 KB, from L2) instead of waiting for a launch that scans
+// them, which took 2 to 4 us: the scan's stage went from 13.7 to 7.7 us for
+// an L = 8 box, 13.7 to 10.8 us at L = 24 and 15.1 to 12.9 us at L = 64
+// (event times, with the gaps between launches).  Beyond that the sums are
+// scanned by one block.
+constexpr int kScanSumTiles = 2048;
+static void launch_scan(const Packed &P, bool advance, cudaStream_t s) {
+  const int nt = scan_tiles(P.ncell);
+  if (nt > 1) k_scan_reduce<<<nt, kScanThreads, 0, s>>>(P.count, P.bsum);
+  if (nt > kScanSumTiles) k_scan_bsum<<<1, 1024, 0, s>>>(P.bsum, nt);
+  k_scan_apply<<<nt, kScanThreads, 0, s>>>(P, advance, nt <= kScanSumTiles);
+}
+
 cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConfig &cfg,
                         cudaStream_t s, bool fused_in, bool fuse_out) {
   if (P.ntot <= 0) return cudaSuccess;
@@ -571,10 +598,7 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
   } else {
     k_integrate_bin<false><<<gb, kBinThreads, 0, s>>>(P, move);
   }
-  const int nt = scan_tiles(P.ncell);
-  k_scan_reduce<<<nt, kScanThreads, 0, s>>>(P.count, P.bsum);
-  k_scan_bsum<<<1, 1024, 0, s>>>(P.bsum, nt);
-  k_scan_apply<<<nt, kScanThreads, 0, s>>>(P, advance);
+  launch_scan(P, advance, s);
   if (cfg.stencil == 1) {
     k_bin_scatter<false><<<gb, kBinThreads, 0, s>>>(P, true);
   } else {
@@ -598,10 +622,7 @@ cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream
   else
     k_integrate_bin<false><<<gb, kBinThreads, 0, s>>>(P, true);
   if ((e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
-  const int nt = scan_tiles(P.ncell);
-  k_scan_reduce<<<nt, kScanThreads, 0, s>>>(P.count, P.bsum);
-  k_scan_bsum<<<1, 1024, 0, s>>>(P.bsum, nt);
-  k_scan_apply<<<nt, kScanThreads, 0, s>>>(P, true);
+  launch_scan(P, true, s);
   if ((e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
   if (cfg.stencil != 1) k_bin_keys<<<gb, kBinThreads, 0, s>>>(P);
   if ((e = cudaEventRecord(ev[3], s)) != cudaSuccess) return e;

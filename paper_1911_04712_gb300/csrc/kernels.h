@@ -259,7 +259,7 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
 cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,
                               cudaEvent_t *ev);
 constexpr int kNumStages = 5;
-constexpr int kKernelsPerStep = 7;
+constexpr int kKernelsPerStep = 6;
 
 // Per-work-item FP64 partial sums for box statistics.
 // With box_out: also the per-box totals (nbox x kStatsFields, a fixed order per box).

@@ -30,7 +30,7 @@ PARAM_NOISE = 12
 PARAM_FUSE = 13
 NOISE_UNIFORM, NOISE_GAUSSIAN = 0, 1
 STENCIL_FULL, STENCIL_HALF = 0, 1
-NUM_STAGES, KERNELS_PER_STEP = 5, 7
+NUM_STAGES, KERNELS_PER_STEP = 5, 6
 
 
 def kernels_per_step(half: bool, force_bands: int = 1) -> int:
