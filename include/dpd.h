@@ -102,7 +102,9 @@ typedef struct dpd_ctx dpd_ctx;
                                      blocks whose neighbourhood exceeds it read global memory */
 
 #define DPD_PARAM_FORCE_VARIANT 11 /* direct force-kernel variant 0..DPD_NUM_FORCE_VARIANTS-1, or -1
-                                      (default) to pick per density band from the tuning table */
+                                      (default) to pick per density band from the tuning table; a
+                                      small single box then runs the row-parallel kernel, with the
+                                      same results (the full stencil's bit for bit) */
 
 #define DPD_PARAM_NOISE 12        /* DPD_NOISE_UNIFORM (default) or DPD_NOISE_GAUSSIAN */
 

@@ -284,6 +284,7 @@ int Engine::build_bands() {
                                  cudaMemcpyHostToDevice, stream_));
   cfg_.mixed_warps = d_mixed_;
   cfg_.hboxes = boxes_.data();
+  cfg_.rows = nb == 1 && variant_override_ < 0;  // a variant asked for is the one that runs
   cfg_.nbands = (int)runs.size();
   for (int k = 0; k < cfg_.nbands; ++k) cfg_.band[k] = runs[k];
   return DPD_OK;

@@ -73,6 +73,69 @@ __device__ __forceinline__ int scan_range(const float4 *__restrict__ pos, int j0
   return -1;
 }
 
+// r_ij of list entry e for a target at qi and its neighbour at pj.
+template <typename BX>
+__device__ __forceinline__ void pair_vector(const BX &B, uint32_t e, const float4 &qi,
+                                            const float4 &pj, float &dx, float &dy, float &dz) {
+  if (e & ~kSlotMask) {  // pair across a box face (rare)
+    const float Lx = B.L[0], Ly = B.L[1], Lz = B.L[2];
+    dx = ((e & kCodeIX) ? qi.x - Lx : qi.x) - ((e & kCodeJX) ? pj.x - Lx : pj.x);
+    dy = ((e & kCodeIY) ? qi.y - Ly : qi.y) - ((e & kCodeJY) ? pj.y - Ly : pj.y);
+    dz = ((e & kCodeIZ) ? qi.z - Lz : qi.z) - ((e & kCodeJZ) ? pj.z - Lz : pj.z);
+  } else {
+    dx = qi.x - pj.x;
+    dy = qi.y - pj.y;
+    dz = qi.z - pj.z;
+  }
+}
+
+// Force of the pair at r_ij = (dx, dy, dz), 0 < r2 = r_ij^2 < rc^2, on i (3),
+// and r . F^C.  wi, wj: the particles' id words; (slo, shi): the noise step.
+template <bool GAUSS, typename BX>
+__device__ __forceinline__ float4 pair_force(const BX &B, float dx, float dy, float dz, float r2,
+                                             const float4 &ui, const float4 &vj, uint32_t wi,
+                                             uint32_t wj, uint32_t slo, uint32_t shi) {
+  // interaction parameters; the general kernels also serve boxes of
+  // several species, whose pair of species picks them (and a cut-off
+  // rc_st <= rc that the pair must be inside)
+  float pa = B.a, pgam = B.gamma, psig = B.sig, psig_g = 0.f, pinv_rc = B.inv_rc;
+  if constexpr (GAUSS) {
+    psig_g = B.sig_g;
+    if (B.nspec > 1) {
+      const int k = (int)((wi >> kSpeciesShift) * kMaxSpecies + (wj >> kSpeciesShift));
+      if (!(r2 < B.sp_rc2[k])) return make_float4(0.f, 0.f, 0.f, 0.f);
+      pa = B.sp_a[k];
+      pgam = B.sp_gamma[k];
+      psig = B.sp_sig[k];
+      psig_g = B.sp_sig_g[k];
+      pinv_rc = B.sp_inv_rc[k];
+    }
+    wi &= kIdMask;  // the pair noise takes the ids alone
+    wj &= kIdMask;
+  }
+  const float rinv = rsqrtf(r2);
+  const float r = r2 * rinv;
+  const float w = fmaxf(fmaf(-r, pinv_rc, 1.0f), 0.0f);
+  const float wR = B.kexp == 1.0f ? w : powf(w, B.kexp);
+  const float ev = fmaf(dx, ui.x - vj.x, fmaf(dy, ui.y - vj.y, dz * (ui.z - vj.z))) * rinv;
+  float fr;  // random term sigma w_R xi / sqrt(dt)
+  if constexpr (GAUSS) {  // general kernels: Gaussian noise or several species
+    const uint2 u = pair_words(wi, wj, slo, shi, B.seed_lo, B.seed_hi);
+    if (B.noise == 0)
+      fr = psig * wR * noise_int(u.x);
+    else
+      fr = psig_g * wR * gauss_xi(u.x, u.y);
+  } else {
+    const uint32_t u = pair_word(wi, wj, slo, shi, B.seed_lo, B.seed_hi);
+    fr = psig * wR * noise_int(u);
+  }
+  const float fc = pa * w;
+  const float s = (fr + fmaf(-pgam * wR * wR, ev, fc)) * rinv;
+  // rounded products (no fusion into the caller's sums), so that every
+  // drain order-preserving variant adds exactly the same terms
+  return make_float4(__fmul_rn(s, dx), __fmul_rn(s, dy), __fmul_rn(s, dz), __fmul_rn(fc, r));
+}
+
 // Per-warp scratch of the balanced drain.  List of lane l: list[l * (CAP+1) + k].
 template <int CAP>
 struct WarpScratch {
@@ -82,6 +145,49 @@ struct WarpScratch {
   float4 res[32];       // pair results of the chunk being processed
   int start[32];        // lane whose list starts at this chunk position, or -1
 };
+
+// The end of a target's force: the body force (Sec. 4.2 periodic Poiseuille,
+// or constant), then the sum is stored, added (half stencil), or, fused with
+// the next step's row a1, used at once.
+template <bool HALF, typename BX>
+__device__ __forceinline__ void finish_force(const Packed &P, const BX &B, const BoxState &S, int p,
+                                             const float4 &pi, const float4 &vi, bool alive,
+                                             bool real, bool fuse, float fx, float fy, float fz,
+                                             float vir) {
+  if (!alive) {
+    // fused step, box not advanced: the next step only bins this slot
+    if constexpr (!HALF) {
+      if (fuse && real)  // stopped box: keeps its slots
+        integrate_one(P, B, p, P.pos[p], P.vel[p], 0.f, 0.f, 0.f, false, false, true);
+    }
+    return;
+  }
+  if (B.fb_mode != 0) {
+    float add = B.fb;
+    if (B.fb_mode == 2) {
+      const float xg = (B.fb_grad == 0) ? pi.x : (B.fb_grad == 1) ? pi.y : pi.z;
+      add = (xg <= B.fb_half) ? -B.fb : B.fb;
+    }
+    if (B.fb_flow == 0)
+      fx += add;
+    else if (B.fb_flow == 1)
+      fy += add;
+    else
+      fz += add;
+  }
+  if constexpr (HALF) {
+    atomicAdd(P.frc + p, make_float4(fx, fy, fz, vir));
+  } else if (fuse) {
+    // the full stencil's force on p is complete here: the next step's row a1
+    // for p, instead of storing the force for a separate integrate pass.  A
+    // box that stops after this step keeps its force for later read-outs.
+    const bool moves = S.remaining > 0;
+    integrate_one(P, B, p, pi, vi, fx, fy, fz, moves, true, !moves);
+    if (!moves) P.frc[p] = make_float4(fx, fy, fz, vir);
+  } else {
+    P.frc[p] = make_float4(fx, fy, fz, vir);
+  }
+}
 
 // Force on one target particle in slot p from the 27-cell (full) or 13-cell
 // + own-cell (half) neighbourhood, each row scanned over the x slices within
@@ -126,7 +232,6 @@ __device__ __forceinline__ void force_direct(const Packed &P, const BX &B, const
   const int xlo = __float2int_rd((pi.x - B.xwin) * B.invh[0]);
   const int xhi = __float2int_rd((pi.x + B.xwin) * B.invh[0]);
   const uint32_t rc2m1 = __float_as_uint(B.rc2) - 1u;
-  const bool k_is_one = (B.kexp == 1.0f);
   if constexpr (SPREAD) {
     own[threadIdx.x & 31] = pi;  // w: id bits
     own[32 + (threadIdx.x & 31)] = vi;
@@ -140,57 +245,10 @@ __device__ __forceinline__ void force_direct(const Packed &P, const BX &B, const
                      const float4 &ui) -> float4 {
     const int j = (int)(e & kSlotMask);
     float dx, dy, dz;
-    if (e & ~kSlotMask) {  // pair across a box face (rare)
-      dx = ((e & kCodeIX) ? qi.x - Lx : qi.x) - ((e & kCodeJX) ? pj.x - Lx : pj.x);
-      dy = ((e & kCodeIY) ? qi.y - Ly : qi.y) - ((e & kCodeJY) ? pj.y - Ly : pj.y);
-      dz = ((e & kCodeIZ) ? qi.z - Lz : qi.z) - ((e & kCodeJZ) ? pj.z - Lz : pj.z);
-    } else {
-      dx = qi.x - pj.x;
-      dy = qi.y - pj.y;
-      dz = qi.z - pj.z;
-    }
+    pair_vector(B, e, qi, pj, dx, dy, dz);
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    // interaction parameters; the general kernels also serve boxes of
-    // several species, whose pair of species picks them (and a cut-off
-    // rc_st <= rc that the pair must be inside)
-    float pa = B.a, pgam = B.gamma, psig = B.sig, psig_g = 0.f, pinv_rc = B.inv_rc;
-    uint32_t idi_ = __float_as_uint(qi.w), idj_ = __float_as_uint(pj.w);
-    if constexpr (GAUSS) {
-      psig_g = B.sig_g;
-      if (B.nspec > 1) {
-        const int k = (int)((idi_ >> kSpeciesShift) * kMaxSpecies + (idj_ >> kSpeciesShift));
-        if (!(r2 < B.sp_rc2[k])) return make_float4(0.f, 0.f, 0.f, 0.f);
-        pa = B.sp_a[k];
-        pgam = B.sp_gamma[k];
-        psig = B.sp_sig[k];
-        psig_g = B.sp_sig_g[k];
-        pinv_rc = B.sp_inv_rc[k];
-      }
-      idi_ &= kIdMask;  // the pair noise takes the ids alone
-      idj_ &= kIdMask;
-    }
-    const float rinv = rsqrtf(r2);
-    const float r = r2 * rinv;
-    const float w = fmaxf(fmaf(-r, pinv_rc, 1.0f), 0.0f);
-    const float wR = k_is_one ? w : powf(w, B.kexp);
-    const float ev = fmaf(dx, ui.x - vj.x, fmaf(dy, ui.y - vj.y, dz * (ui.z - vj.z))) * rinv;
-    float fr;  // random term sigma w_R xi / sqrt(dt)
-    if constexpr (GAUSS) {  // general kernels: Gaussian noise or several species
-      const uint2 u = pair_words(idi_, idj_, slo, shi, B.seed_lo, B.seed_hi);
-      if (B.noise == 0)
-        fr = psig * wR * noise_int(u.x);
-      else
-        fr = psig_g * wR * gauss_xi(u.x, u.y);
-    } else {
-      const uint32_t u = pair_word(idi_, idj_, slo, shi, B.seed_lo, B.seed_hi);
-      fr = psig * wR * noise_int(u);
-    }
-    const float fc = pa * w;
-    const float s = (fr + fmaf(-pgam * wR * wR, ev, fc)) * rinv;
-    // rounded products (no fusion into the caller's sums), so that every
-    // drain order-preserving variant adds exactly the same terms
-    const float4 g = make_float4(__fmul_rn(s, dx), __fmul_rn(s, dy), __fmul_rn(s, dz),
-                                 __fmul_rn(fc, r));
+    const float4 g = pair_force<GAUSS>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
+                                       __float_as_uint(pj.w), slo, shi);
     if constexpr (HALF) atomicAdd(P.frc + j, make_float4(-g.x, -g.y, -g.z, g.w));
     return g;
   };
@@ -452,39 +510,7 @@ __device__ __forceinline__ void force_direct(const Packed &P, const BX &B, const
   }
   drain();
 
-  if (!alive) {
-    // fused step, box not advanced: the next step only bins this slot
-    if constexpr (!HALF) {
-      if (fuse && real)  // stopped box: keeps its slots
-        integrate_one(P, B, p, P.pos[p], P.vel[p], 0.f, 0.f, 0.f, false, false, true);
-    }
-    return;
-  }
-  if (B.fb_mode != 0) {  // body force (Sec. 4.2 periodic Poiseuille, or constant)
-    float add = B.fb;
-    if (B.fb_mode == 2) {
-      const float xg = (B.fb_grad == 0) ? pi.x : (B.fb_grad == 1) ? pi.y : pi.z;
-      add = (xg <= B.fb_half) ? -B.fb : B.fb;
-    }
-    if (B.fb_flow == 0)
-      fx += add;
-    else if (B.fb_flow == 1)
-      fy += add;
-    else
-      fz += add;
-  }
-  if constexpr (HALF) {
-    atomicAdd(P.frc + p, make_float4(fx, fy, fz, vir));
-  } else if (fuse) {
-    // the full stencil's force on p is complete here: the next step's row a1
-    // for p, instead of storing the force for a separate integrate pass.  A
-    // box that stops after this step keeps its force for later read-outs.
-    const bool moves = S.remaining > 0;
-    integrate_one(P, B, p, pi, vi, fx, fy, fz, moves, true, !moves);
-    if (!moves) P.frc[p] = make_float4(fx, fy, fz, vir);
-  } else {
-    P.frc[p] = make_float4(fx, fy, fz, vir);
-  }
+  finish_force<HALF>(P, B, S, p, pi, vi, alive, real, fuse, fx, fy, fz, vir);
 }
 
 }  // namespace dpd

@@ -1,0 +1,260 @@
+// Row-parallel force kernels for small sets (pair forces, Sec. 2.1 Eqs. 2-5,
+// over the cell list of Sec. 3.2).  A block owns 32 target slots and has one
+// warp per stencil row: warp r scans row r for the 32 targets at once, the
+// lists of all rows are gathered into one queue, every thread of the block
+// evaluates pairs of the queue, and with the full stencil each target then
+// adds its pairs' results in row and slot order: the order, and so the bits,
+// of the direct routine.
+//
+// What bounds it: latency.  A set of a few thousand particles is a handful
+// of warps per SM, and the direct routine has each of them walk nine rows
+// and evaluate up to twenty pairs one after the other, most of the time
+// waiting for one load.  Here a step's chain is one row scan, about two pair
+// evaluations and one ordered sum.  Force stage at rho = 3, direct against
+// row-parallel: N = 1,536 full 28.6 -> 10.2 us, half 18.4 -> 8.2; N = 55,296
+// (rho = 4) full 41.3 -> 33.1, half 23.9 -> 18.3.  launch_force says where the
+// lines cross.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "dpd_device.cuh"
+#include "force_direct.cuh"
+#include "kernels.h"
+
+namespace dpd {
+
+namespace {
+
+constexpr int kRowsUnroll = 8;  // candidates loaded per iteration: a row's window at rho = 3
+constexpr int kRowsCap = 40;    // list places of one target in one row
+constexpr unsigned kAll = 0xffffffffu;
+
+template <bool HALF>
+struct RowsShared {
+  static constexpr int kRows = HALF ? 5 : 9, kThreads = 32 * kRows;
+  static constexpr int kQueue = HALF ? 1536 : 2880;
+  float4 own_pos[32], own_vel[32];
+  union {
+    uint32_t list[kRowsCap * kThreads];  // entry k of thread t at k * kThreads + t
+    float4 res[HALF ? 1 : kQueue];       // after the lists were gathered
+  };
+  uint32_t queue[kQueue];                // list entries: rows in order, lanes in order
+  uint8_t who[kQueue];                   // their targets' lanes
+  uint16_t off[kRows][32], cnt[kRows][32];
+  int row_total[kRows];
+  int overflow;
+};
+
+template <bool HALF, bool GAUSS>
+__global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
+    k_force_rows(Packed P, bool fuse) {
+  using Sh = RowsShared<HALF>;
+  constexpr int NT = Sh::kThreads, U = kRowsUnroll, CAP = kRowsCap;
+  extern __shared__ float4 rows_smem[];
+  Sh &W = *reinterpret_cast<Sh *>(rows_smem);
+  const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
+  const int p0 = (int)blockIdx.x * 32, p = p0 + lane;
+  const bool real = p < P.ntot;
+  const BoxDev &B = P.single;
+  const BoxState S = P.st[0];
+  const bool alive = real && S.adv && DPD_IN_BOUNDS(p >= 0 && p < P.ntot, P.err);
+  float4 pi = make_float4(0.f, 0.f, 0.f, 0.f), vi = pi;
+  if (alive) {
+    pi = P.pos[p];
+    vi = P.vel[p];
+  }
+  if (row == 0) {
+    W.own_pos[lane] = pi;
+    W.own_vel[lane] = vi;
+  }
+  if (tid == 0) W.overflow = 0;
+
+  // ---- this warp's row (rows as in the direct routine)
+  int cnt = 0;
+  bool over = false;
+  if (alive) {
+    const int dz = HALF ? (row < 2 ? 0 : 1) : row / 3 - 1;
+    const int dy = HALF ? (row == 0 ? 0 : (row == 1 ? 1 : row - 3)) : row - 3 * (row / 3) - 1;
+    const float Lx = B.L[0], Ly = B.L[1], Lz = B.L[2];
+    const int nx = B.n[0], ny = B.n[1], nz = B.n[2];
+    int cx, cy, cz;
+    unpack_cell(__float_as_int(vi.w), cx, cy, cz);
+    const int xlo = __float2int_rd((pi.x - B.xwin) * B.invh[0]);
+    const int xhi = __float2int_rd((pi.x + B.xwin) * B.invh[0]);
+    int z = cz + dz, y = cy + dy;
+    float az = pi.z, jsz = 0.f, ay = pi.y, jsy = 0.f;
+    uint32_t code = 0;
+    if (z < 0) {
+      z += nz;
+      jsz = Lz;
+      code |= kCodeJZ;
+    } else if (z >= nz) {
+      z -= nz;
+      az = pi.z - Lz;
+      code |= kCodeIZ;
+    }
+    if (y < 0) {
+      y += ny;
+      jsy = Ly;
+      code |= kCodeJY;
+    } else if (y >= ny) {
+      y -= ny;
+      ay = pi.y - Ly;
+      code |= kCodeIY;
+    }
+    const int rowbase = B.cellBase + (z * ny + y) * nx;
+    const bool own = HALF && row == 0;
+    const int lo = own ? cx : xlo, hi = xhi;
+    if (DPD_IN_BOUNDS(rowbase >= 0 && rowbase + nx <= P.ncell && lo >= -nx && lo <= hi &&
+                          hi < 2 * nx, P.err)) {
+      const int nseg = (lo < 0 || hi >= nx) ? 2 : 1;
+      // both ends of both parts at once: [s0, s1) and, across an x face, [0, s2)
+      const int s0 = lo < 0 ? lo + nx : lo, s1 = (lo < 0 || hi >= nx) ? nx : hi + 1;
+      const int s2 = lo < 0 ? hi + 1 : hi - nx + 1;
+      int j0 = own ? p + 1 : __ldg(P.start + rowbase + s0);
+      int j1 = __ldg(P.start + rowbase + s1);
+      int k0 = 0, k1 = 0;
+      if (nseg == 2) {
+        k0 = __ldg(P.start + rowbase);
+        k1 = __ldg(P.start + rowbase + s2);
+      }
+      if (!DPD_IN_BOUNDS(j0 >= 0 && j0 <= j1 && j1 <= P.ntot && k0 >= 0 && k0 <= k1 &&
+                             k1 <= P.ntot, P.err))
+        j0 = j1 = k0 = k1 = 0;
+      const uint32_t rc2m1 = __float_as_uint(B.rc2) - 1u;
+#pragma unroll 1
+      for (int sg = 0; sg < nseg && !over; ++sg) {
+        float ax = pi.x, jsx = 0.f;
+        uint32_t c = code;
+        int a0 = j0, a1 = j1;
+        if (lo < 0) {  // slices lo + nx .. nx - 1 as r_j - L, then 0 .. hi
+          if (sg == 0) {
+            jsx = Lx;
+            c |= kCodeJX;
+          } else {
+            a0 = k0;
+            a1 = k1;
+          }
+        } else if (sg == 1) {  // lo .. nx - 1, then 0 .. hi - nx seen from r_i - L
+          a0 = k0;
+          a1 = k1;
+          ax = pi.x - Lx;
+          c |= kCodeIX;
+        }
+        const int stop = scan_range<true, NT, CAP, U>(P.pos, a0, a1, ax, ay, az, jsx, jsy, jsz,
+                                                      rc2m1, c, W.list + tid, cnt);
+        over = stop >= 0 && (stop < a1 || sg + 1 < nseg);
+      }
+    }
+  }
+
+  // ---- places in the queue: rows in order, lanes in order
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kAll, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) W.row_total[row] = incl;
+  __syncthreads();
+  if (over) W.overflow = 1;
+  int base = 0, total = 0;
+#pragma unroll
+  for (int r = 0; r < Sh::kRows; ++r) {
+    const int n = W.row_total[r];
+    base += r < row ? n : 0;
+    total += n;
+  }
+  const int off = base + incl - cnt;
+  W.off[row][lane] = (uint16_t)off;
+  W.cnt[row][lane] = (uint16_t)cnt;
+  if (total <= Sh::kQueue)
+    for (int k = 0; k < cnt; ++k) {
+      W.queue[off + k] = W.list[k * NT + tid];
+      W.who[off + k] = (uint8_t)lane;
+    }
+  __syncthreads();
+
+  if (W.overflow || total > Sh::kQueue) {
+    // a denser place than the lists hold: the direct routine, by one warp
+    if (row == 0)
+      force_direct<HALF, NT, CAP, false, GAUSS>(P, P.single, S, p, alive, W.list + tid, nullptr,
+                                                nullptr, false, fuse, real);
+    return;
+  }
+
+  // ---- evaluate the queue
+#pragma unroll 1
+  for (int q = tid; q < total; q += NT) {
+    const uint32_t e = W.queue[q];
+    const int o = W.who[q], j = (int)(e & kSlotMask);
+    if (!DPD_IN_BOUNDS(j < P.ntot, P.err)) continue;
+    const float4 pj = __ldg(P.pos + j), vj = __ldg(P.vel + j);
+    const float4 qi = W.own_pos[o], ui = W.own_vel[o];
+    float dx, dy, dz;
+    pair_vector(B, e, qi, pj, dx, dy, dz);
+    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float4 g = pair_force<GAUSS>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
+                                       __float_as_uint(pj.w), (uint32_t)S.step,
+                                       (uint32_t)(S.step >> 32));
+    if constexpr (HALF) {
+      atomicAdd(P.frc + j, make_float4(-g.x, -g.y, -g.z, g.w));
+      atomicAdd(P.frc + (p0 + o), g);
+    } else {
+      W.res[q] = g;
+    }
+  }
+
+  if constexpr (!HALF) __syncthreads();
+  if (row != 0) return;
+  float fx = 0.f, fy = 0.f, fz = 0.f, vir = 0.f;
+  if constexpr (!HALF) {
+#pragma unroll 1
+    for (int r = 0; r < Sh::kRows; ++r) {
+      const int q0 = W.off[r][lane], q1 = q0 + W.cnt[r][lane];
+#pragma unroll 4
+      for (int q = q0; q < q1; ++q) {
+        const float4 g = W.res[q];
+        fx += g.x;
+        fy += g.y;
+        fz += g.z;
+        vir += g.w;
+      }
+    }
+  }
+  finish_force<HALF>(P, B, S, p, pi, vi, alive, real, fuse, fx, fy, fz, vir);
+}
+
+template <bool HALF, bool GAUSS>
+cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s) {
+  using Sh = RowsShared<HALF>;
+  k_force_rows<HALF, GAUSS><<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse);
+  return cudaGetLastError();
+}
+
+template <bool HALF, bool GAUSS>
+cudaError_t prepare_one() {
+  return cudaFuncSetAttribute(k_force_rows<HALF, GAUSS>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(RowsShared<HALF>));
+}
+
+}  // namespace
+
+cudaError_t prepare_rows() {
+  cudaError_t e = prepare_one<false, false>();
+  if (e == cudaSuccess) e = prepare_one<false, true>();
+  if (e == cudaSuccess) e = prepare_one<true, false>();
+  if (e == cudaSuccess) e = prepare_one<true, true>();
+  return e;
+}
+
+cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse,
+                              cudaStream_t s) {
+  if (P.nbox != 1 || (fuse && half)) return cudaErrorInvalidValue;
+  if (half) return general ? launch_one<true, true>(P, fuse, s) : launch_one<true, false>(P, fuse, s);
+  return general ? launch_one<false, true>(P, fuse, s) : launch_one<false, false>(P, fuse, s);
+}
+
+}  // namespace dpd

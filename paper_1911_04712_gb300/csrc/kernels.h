@@ -123,6 +123,7 @@ struct StepConfig {
   const int *mixed_warps = nullptr;  // device: first slots of the bands' two-box warps
   BrickGrid bricks{};                // work items of the brick force kernel
   const BoxDev *hboxes = nullptr;    // host copies of the box constants (grouped launches)
+  bool rows = false;                 // one box: the row-parallel kernels where they pay
   bool grouped = true;               // packed half stencil: box-grouped launches
 };
 // Whether the variant drains over the whole warp (balanced or spread): such
@@ -136,6 +137,10 @@ size_t tile_smem_bytes(int stage_cap);
 // (integrate_one) for every slot and stores no force.
 cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
                          bool fuse = false);
+
+// Row-parallel force kernels of one small box (force_rows.cu).
+cudaError_t prepare_rows();
+cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s);
 
 // Direct force-kernel variants (threads per block, pair-list capacity).
 int force_variant_info(int v, int *threads, int *cap);

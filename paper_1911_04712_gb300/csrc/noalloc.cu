@@ -90,8 +90,9 @@ static unsigned char *scratch_address(int device, int *status) {
   if (!addr[device]) {
     void *p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+    if (e == cudaSuccess) e = prepare_device();  // launch attributes of the force kernels
     if (e != cudaSuccess || !p) {
-      *status = set_error(DPD_ERR_CUDA, "cudaGetSymbolAddress(scratch): %s",
+      *status = set_error(DPD_ERR_CUDA, "preparing dpd_forces_noalloc: %s",
                           cudaGetErrorString(e));
       return nullptr;
     }
@@ -172,6 +173,7 @@ extern "C" int dpd_forces_noalloc(int64_t n, const float *pos, const float *vel,
   DPD_CUDA_TRY(cudaGetLastError());
   DPD_CUDA_TRY(launch_load(P, 0, (int)n, pos, vel, P.single.L[0], P.single.L[1], P.single.L[2], s));
   StepConfig cfg{};
+  cfg.rows = true;
   DPD_CUDA_TRY(launch_step(P, false, false, cfg, s));
   DPD_CUDA_TRY(launch_gather(P, 0, 0, (int)n, nullptr, nullptr, force, s));
 #if defined(DPD_CHECKED) && DPD_CHECKED
