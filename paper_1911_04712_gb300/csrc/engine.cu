@@ -11,6 +11,9 @@
 
 namespace dpd {
 
+// Sets up to this size replay a call's last steps from graphs (Engine::step).
+constexpr int kGraphTailSlots = 131072;
+
 static thread_local std::string t_err;
 
 int set_error(int code, const char *fmt, ...) {
@@ -442,11 +445,12 @@ int Engine::build_bricks() {
 }
 
 void Engine::drop_graph() {
-  for (cudaGraphExec_t *g : {&graph_, &graph1_})
-    if (*g) {
-      cudaGraphExecDestroy(*g);
-      *g = nullptr;
-    }
+  auto drop = [](cudaGraphExec_t &g) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  };
+  drop(graph_);
+  for (cudaGraphExec_t &g : tail_) drop(g);
 }
 
 int Engine::free_all() {
@@ -693,6 +697,22 @@ int Engine::capture_graph(int nsteps, cudaGraphExec_t *out) {
   return DPD_OK;
 }
 
+int Engine::launch_graph(cudaGraphExec_t *g, int nsteps) {
+  if (!*g) {
+    int rc = capture_graph(nsteps, g);
+    if (rc) return rc;
+  }
+  DPD_CUDA_TRY(cudaGraphLaunch(*g, stream_));
+  return DPD_OK;
+}
+
+bool Engine::capturing() const {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream_, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy default stream beside a capture elsewhere
+  return true;
+}
+
 int Engine::step(int64_t nsteps) {
   NvtxRange range("dpd step");
   if (nsteps < 0) return set_error(DPD_ERR_ARG, "nsteps must be >= 0");
@@ -710,24 +730,19 @@ int Engine::step(int64_t nsteps) {
     return DPD_OK;
   }
   int64_t left = nsteps;
-  if (graph_chunk > 1 && left >= graph_chunk) {
-    if (!graph_) {
-      int rc = capture_graph(graph_chunk, &graph_);
-      if (rc) return rc;
-    }
-    while (left >= graph_chunk) {
-      DPD_CUDA_TRY(cudaGraphLaunch(graph_, stream_));
-      left -= graph_chunk;
-    }
-  }
-  if (left == 1 && graph_chunk > 1) {  // one step: a cached one-step graph, one launch
-    if (!graph1_) {
-      int rc = capture_graph(1, &graph1_);
-      if (rc) return rc;
-    }
-    DPD_CUDA_TRY(cudaGraphLaunch(graph1_, stream_));
-    left = 0;
-  }
+  int rc = DPD_OK;
+  for (; graph_chunk > 1 && left >= graph_chunk; left -= graph_chunk)
+    if ((rc = launch_graph(&graph_, graph_chunk))) return rc;
+  // The rest: one step is a graph of its own.  Several steps are graphs of
+  // 2^k steps where the host launches kernels (about 7 us each) slower than
+  // they run: 20 steps of an L = 24 box took 769 us by direct launches, 547
+  // by graphs, and the first call, which captures them, 792 -> 590 us
+  // (N = 41,472).  At 98,304 slots 20 steps went from 1226 to 941 us; from
+  // 140,000 on the launches keep up and steps start sooner without a capture.
+  if (graph_chunk > 1 && (left == 1 || (left > 1 && ntot_ <= kGraphTailSlots && !capturing())))
+    for (int k = kTails - 1; k >= 0; --k)
+      for (; left >= (int64_t)1 << k; left -= (int64_t)1 << k)
+        if ((rc = launch_graph(&tail_[k], 1 << k))) return rc;
   const Packed P = packed();
   const bool fz = fused_steps();  // the last step of the call stays plain: read-outs follow
   for (int64_t k = 0; k < left; ++k) {

@@ -228,7 +228,11 @@ class Engine {
   int ensure_sampling_buffers();
   int launch_extra(const Packed &P, cudaStream_t s);
   cudaGraphExec_t graph_ = nullptr;   // graph_chunk steps
-  cudaGraphExec_t graph1_ = nullptr;  // one step (calls that end with a single step)
+  // 2^k steps: what a call leaves after its whole chunks
+  static constexpr int kTails = 5;
+  cudaGraphExec_t tail_[kTails] = {};
+  int launch_graph(cudaGraphExec_t *g, int nsteps);
+  bool capturing() const;  // the caller's stream is being captured
 };
 
 }  // namespace dpd
