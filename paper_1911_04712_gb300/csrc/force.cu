@@ -462,7 +462,7 @@ cudaError_t prepare_device() {
 // 98,304 (rho 3).  Above about 12 particles per cell the lists of a row
 // would often overflow (the kernels then fall back to the direct routine).
 constexpr int kRowsMaxFull = 65536, kRowsMaxHalf = 98304, kRowsMaxPerCell = 12;
-static bool rows_pay(const Packed &P, bool half) {
+bool rows_pay(const Packed &P, bool half) {
   return P.nbox == 1 && P.ntot <= (half ? kRowsMaxHalf : kRowsMaxFull) &&
          (long long)P.ntot * kSlicesX <= (long long)kRowsMaxPerCell * P.ncell;
 }

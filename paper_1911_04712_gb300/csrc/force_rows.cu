@@ -46,9 +46,18 @@ struct RowsShared {
   int overflow;
 };
 
+// A force to its particle's place in an n x 3 array.
+__device__ __forceinline__ void store3(float *__restrict__ out3, const float4 &pi,
+                                       const float4 &f) {
+  float *o = out3 + 3 * (size_t)(__float_as_uint(pi.w) & kIdMask);
+  o[0] = f.x;
+  o[1] = f.y;
+  o[2] = f.z;
+}
+
 template <bool HALF, bool GAUSS>
 __global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
-    k_force_rows(Packed P, bool fuse) {
+    k_force_rows(Packed P, bool fuse, float *__restrict__ out3) {
   using Sh = RowsShared<HALF>;
   constexpr int NT = Sh::kThreads, U = kRowsUnroll, CAP = kRowsCap;
   extern __shared__ float4 rows_smem[];
@@ -178,9 +187,11 @@ __global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
 
   if (W.overflow || total > Sh::kQueue) {
     // a denser place than the lists hold: the direct routine, by one warp
-    if (row == 0)
+    if (row == 0) {
       force_direct<HALF, NT, CAP, false, GAUSS>(P, P.single, S, p, alive, W.list + tid, nullptr,
                                                 nullptr, false, fuse, real);
+      if (out3 && alive) store3(out3, pi, P.frc[p]);
+    }
     return;
   }
 
@@ -224,12 +235,13 @@ __global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
     }
   }
   finish_force<HALF>(P, B, S, p, pi, vi, alive, real, fuse, fx, fy, fz, vir);
+  if (out3 && alive) store3(out3, pi, P.frc[p]);  // this thread's own store
 }
 
 template <bool HALF, bool GAUSS>
-cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s) {
+cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
   using Sh = RowsShared<HALF>;
-  k_force_rows<HALF, GAUSS><<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse);
+  k_force_rows<HALF, GAUSS><<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse, out3);
   return cudaGetLastError();
 }
 
@@ -250,11 +262,14 @@ cudaError_t prepare_rows() {
   return e;
 }
 
-cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse,
-                              cudaStream_t s) {
-  if (P.nbox != 1 || (fuse && half)) return cudaErrorInvalidValue;
-  if (half) return general ? launch_one<true, true>(P, fuse, s) : launch_one<true, false>(P, fuse, s);
-  return general ? launch_one<false, true>(P, fuse, s) : launch_one<false, false>(P, fuse, s);
+cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s,
+                              float *out3) {
+  if (P.nbox != 1 || (half && (fuse || out3))) return cudaErrorInvalidValue;
+  if (half)
+    return general ? launch_one<true, true>(P, fuse, s, out3)
+                   : launch_one<true, false>(P, fuse, s, out3);
+  return general ? launch_one<false, true>(P, fuse, s, out3)
+                 : launch_one<false, false>(P, fuse, s, out3);
 }
 
 }  // namespace dpd

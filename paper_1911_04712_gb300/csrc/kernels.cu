@@ -39,29 +39,7 @@ __global__ void k_load(Packed P, int slot0, int n, const float *__restrict__ pos
                        const int32_t *__restrict__ species, int nspec) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  float x[3] = {pos3[3 * i], pos3[3 * i + 1], pos3[3 * i + 2]};
-  const float L[3] = {Lx, Ly, Lz};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    float y = x[k];
-    if (!(y >= 0.0f && y < L[k])) {
-      y = y - L[k] * floorf(y / L[k]);
-      if (y >= L[k]) y = 0.0f;
-      if (!(y >= 0.0f)) {  // NaN or still negative after rounding
-        if (!(y == y)) atomicOr(P.err, kErrNonFinite);
-        y = 0.0f;
-      }
-    }
-    x[k] = y;
-  }
-  int s = species ? species[i] : 0;
-  if (s < 0 || s >= nspec) {
-    atomicOr(P.err, kErrSpecies);
-    s = 0;
-  }
-  P.pos[slot0 + i] =
-      make_float4(x[0], x[1], x[2], __uint_as_float((uint32_t)i | ((uint32_t)s << kSpeciesShift)));
-  P.vel[slot0 + i] = make_float4(vel3[3 * i], vel3[3 * i + 1], vel3[3 * i + 2], 0.0f);
+  load_particle(P, i, pos3, vel3, Lx, Ly, Lz, species, nspec, P.pos[slot0 + i], P.vel[slot0 + i]);
 }
 
 // ------------------------------------------------------- integrate + count
@@ -205,46 +183,13 @@ __global__ void __launch_bounds__(kScanThreads)
 // ---------------------------------------------------------------- reorder
 __global__ void __launch_bounds__(kBinThreads) k_bin_keys(Packed P) {
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
-  if (p >= P.ntot) return;
-  const int c = P.cellOf[p];
-  if (c < 0) return;  // keeps its slot (stopped box): every particle of its cell does
-  if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
-  const int k = P.start[c] + P.slotIn[p];
-  if (!DPD_IN_BOUNDS(k >= 0 && k < P.ntot, P.err)) return;
-  P.keyTmp[k] = p;
+  if (p < P.ntot) bin_key(P, p);
 }
 
-// STABLE: a particle's place in its cell is its rank by previous slot among
-// the cell's particles (listed by k_bin_keys), so the order, and with it the
-// full stencil's sums, are reproducible.  Otherwise (half stencil, whose sums
-// are atomic anyway) it is its arrival rank from the count, as in Sec. 3.2.
-// A particle of a stopped box keeps its slot, and its force (which the half
-// stencil's reorder otherwise clears for the atomic sums): it did not move,
-// so its cell's slot range is the one it was placed in.
 template <bool STABLE>
 __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(Packed P, bool zero_frc) {
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
-  if (p >= P.ntot) return;
-  const int ce = P.cellOf[p];
-  const bool keep = ce < 0;
-  const int c = ce & ~kKeepSlot;
-  if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
-  const int s0 = P.start[c];
-  int dst = p;
-  if (!keep) {
-    int rank = P.slotIn[p];
-    if constexpr (STABLE) {
-      const int s1 = P.start[c + 1];
-      if (!DPD_IN_BOUNDS(s0 >= 0 && s0 <= s1 && s1 <= P.ntot, P.err)) return;
-      rank = 0;
-      for (int t = s0; t < s1; ++t) rank += (P.keyTmp[t] < p) ? 1 : 0;
-    }
-    dst = s0 + rank;
-  }
-  if (!DPD_IN_BOUNDS(dst >= s0 && dst < P.start[c + 1] && dst < P.ntot, P.err)) return;
-  P.pos[dst] = P.pos2[p];
-  P.vel[dst] = P.vel2[p];
-  if (zero_frc && !keep) P.frc[dst] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (p < P.ntot) bin_scatter<STABLE>(P, p, zero_frc);
 }
 
 // ------------------------------------------------------------------ stats

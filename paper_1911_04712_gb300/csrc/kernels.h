@@ -140,7 +140,10 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
 
 // Row-parallel force kernels of one small box (force_rows.cu).
 cudaError_t prepare_rows();
-cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s);
+// out3: also write the forces to id order (n x 3, full stencil).
+cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s,
+                              float *out3 = nullptr);
+bool rows_pay(const Packed &P, bool half);  // whether they serve this box
 
 // Direct force-kernel variants (threads per block, pair-list capacity).
 int force_variant_info(int v, int *threads, int *cap);
@@ -217,6 +220,77 @@ __device__ __forceinline__ void integrate_one(const Packed &P, const BX &B, int 
   P.slotIn[p] = atomicAdd(P.count + c, 1);
 }
 
+// Particle i of n x 3 inputs as a slot's records, wrapped into the box.
+__device__ __forceinline__ void load_particle(const Packed &P, int i, const float *__restrict__ pos3,
+                                              const float *__restrict__ vel3, float Lx, float Ly,
+                                              float Lz, const int32_t *__restrict__ species,
+                                              int nspec, float4 &pos, float4 &vel) {
+  float x[3] = {pos3[3 * i], pos3[3 * i + 1], pos3[3 * i + 2]};
+  const float L[3] = {Lx, Ly, Lz};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    float y = x[k];
+    if (!(y >= 0.0f && y < L[k])) {
+      y = y - L[k] * floorf(y / L[k]);
+      if (y >= L[k]) y = 0.0f;
+      if (!(y >= 0.0f)) {  // NaN or still negative after rounding
+        if (!(y == y)) atomicOr(P.err, kErrNonFinite);
+        y = 0.0f;
+      }
+    }
+    x[k] = y;
+  }
+  int s = species ? species[i] : 0;
+  if (s < 0 || s >= nspec) {
+    atomicOr(P.err, kErrSpecies);
+    s = 0;
+  }
+  pos = make_float4(x[0], x[1], x[2], __uint_as_float((uint32_t)i | ((uint32_t)s << kSpeciesShift)));
+  vel = make_float4(vel3[3 * i], vel3[3 * i + 1], vel3[3 * i + 2], 0.0f);
+}
+
+// The reorder's key pass (full stencil): slot p's index at its arrival position.
+__device__ __forceinline__ void bin_key(const Packed &P, int p) {
+  const int c = P.cellOf[p];
+  if (c < 0) return;  // keeps its slot (stopped box): every particle of its cell does
+  if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
+  const int k = P.start[c] + P.slotIn[p];
+  if (!DPD_IN_BOUNDS(k >= 0 && k < P.ntot, P.err)) return;
+  P.keyTmp[k] = p;
+}
+
+// Move slot p to its place in cell order.
+// STABLE: a particle's place in its cell is its rank by previous slot among
+// the cell's particles (listed by k_bin_keys), so the order, and with it the
+// full stencil's sums, are reproducible.  Otherwise (half stencil, whose sums
+// are atomic anyway) it is its arrival rank from the count, as in Sec. 3.2.
+// A particle of a stopped box keeps its slot, and its force (which the half
+// stencil's reorder otherwise clears for the atomic sums): it did not move,
+// so its cell's slot range is the one it was placed in.
+template <bool STABLE>
+__device__ __forceinline__ void bin_scatter(const Packed &P, int p, bool zero_frc) {
+  const int ce = P.cellOf[p];
+  const bool keep = ce < 0;
+  const int c = ce & ~kKeepSlot;
+  if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
+  const int s0 = P.start[c];
+  int dst = p;
+  if (!keep) {
+    int rank = P.slotIn[p];
+    if constexpr (STABLE) {
+      const int s1 = P.start[c + 1];
+      if (!DPD_IN_BOUNDS(s0 >= 0 && s0 <= s1 && s1 <= P.ntot, P.err)) return;
+      rank = 0;
+      for (int t = s0; t < s1; ++t) rank += (P.keyTmp[t] < p) ? 1 : 0;
+    }
+    dst = s0 + rank;
+  }
+  if (!DPD_IN_BOUNDS(dst >= s0 && dst < P.start[c + 1] && dst < P.ntot, P.err)) return;
+  P.pos[dst] = P.pos2[p];
+  P.vel[dst] = P.vel2[p];
+  if (zero_frc && !keep) P.frc[dst] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // Box constants: the kernel parameter copy for a single box, else from memory.
 template <bool SINGLE>
 __device__ __forceinline__ BoxDev box_of(const Packed &P, int b) {
@@ -238,7 +312,9 @@ constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;  // cells per scan tile
 constexpr int kScanMaxTiles = 1024 * 16;              // one block scans up to this many tile sums
 
-inline int scan_tiles(int ncell) { return (ncell + 1 + kScanTile - 1) / kScanTile; }
+inline __host__ __device__ int scan_tiles(int ncell) {
+  return (ncell + 1 + kScanTile - 1) / kScanTile;
+}
 
 // Set per-function launch attributes on the current device (once per device,
 // before any capture).

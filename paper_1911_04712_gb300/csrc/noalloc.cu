@@ -19,6 +19,7 @@
 // start of each call.  Calls whose work overlaps on the GPU (different
 // streams, or different host threads) race on the array and must be
 // serialised by the caller.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -28,6 +29,8 @@
 #include "dpd.h"
 #include "engine.h"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace dpd {
 
@@ -60,20 +63,91 @@ constexpr size_t kScratchBytes = kOffErr + align256(sizeof(unsigned));
 // The scratch: about 3.5 MB for 32768 particles and 32767 cells (two x slices each).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
-// Zero the cell counts and the error word; set the step of the force.
-__global__ void k_noalloc_reset(int ncell_padded, unsigned long long step) {
-  int *count = reinterpret_cast<int *>(g_noalloc_scratch + kOffCount);
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell_padded;
-       c += gridDim.x * blockDim.x)
-    count[c] = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    BoxState *st = reinterpret_cast<BoxState *>(g_noalloc_scratch + kOffState);
-    st->step = step;
-    st->remaining = 0;
-    st->pending = 0;
-    st->adv = 1;
-    *reinterpret_cast<unsigned *>(g_noalloc_scratch + kOffErr) = 0u;
+// The whole rebuild of one call in one launch: counts and error word cleared,
+// the inputs loaded and counted (Sec. 3.2), scan, keys and reorder, by one
+// thread-block cluster whose barriers stand where the separate kernels have
+// launches.  What bounds a call is launches: for n = 1,536 eight or nine small
+// kernels on a stream took 35 us and the host 20 us to launch them; this one
+// and the force kernel take 20.5 and 5.4 us.
+constexpr int kNaBlocks = 8;  // the portable cluster size
+constexpr int kNaThreads = 1024;
+constexpr int kNaAll = kNaBlocks * kNaThreads;
+constexpr int kNaQuads = (int)(kNaCellCap / 4 + kNaAll - 1) / kNaAll;  // per thread, at most
+
+__global__ void __cluster_dims__(kNaBlocks, 1, 1) __launch_bounds__(kNaThreads, 1)
+    k_noalloc_bin(Packed P, const float *__restrict__ pos3, const float *__restrict__ vel3,
+                  unsigned long long step) {
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ int wsum[32];
+  __shared__ int block_total;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int gt = (int)blockIdx.x * kNaThreads + tid;
+  const int quads_all = scan_tiles(P.ncell) * (kScanTile / 4);
+  const int quads = (quads_all + kNaAll - 1) / kNaAll;  // a run of cells per thread
+  int4 *c4 = reinterpret_cast<int4 *>(P.count) + (size_t)gt * quads;
+  int4 *s4 = reinterpret_cast<int4 *>(P.start) + (size_t)gt * quads;
+  for (int k = 0; k < quads && gt * quads + k < quads_all; ++k) c4[k] = make_int4(0, 0, 0, 0);
+  if (gt == 0) {
+    *P.st = BoxState{step, 0ll, 0, 1};
+    *P.err = 0u;
   }
+  cluster.sync();
+
+  const BoxDev &B = P.single;
+  for (int i = gt; i < P.ntot; i += kNaAll) {
+    float4 x, v;
+    load_particle(P, i, pos3, vel3, B.L[0], B.L[1], B.L[2], nullptr, 1, x, v);
+    integrate_one(P, B, i, x, v, 0.f, 0.f, 0.f, false, false);
+  }
+  cluster.sync();
+
+  // exclusive scan of the counts
+  int4 q[kNaQuads];
+  int sum = 0;
+#pragma unroll
+  for (int k = 0; k < kNaQuads; ++k) {
+    q[k] = make_int4(0, 0, 0, 0);
+    if (k < quads && gt * quads + k < quads_all) q[k] = c4[k];
+    sum += q[k].x + q[k].y + q[k].z + q[k].w;
+  }
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  if (warp == 0) {
+    int w = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += t;
+    }
+    wsum[lane] = w;
+    if (lane == 31) block_total = w;
+  }
+  cluster.sync();
+  int other = 0;  // totals of the blocks before this one
+  if (lane < (int)cluster.block_rank()) other = *cluster.map_shared_rank(&block_total, lane);
+  int run = incl - sum + (warp > 0 ? wsum[warp - 1] : 0) + __reduce_add_sync(0xffffffffu, other);
+#pragma unroll
+  for (int k = 0; k < kNaQuads; ++k)
+    if (k < quads && gt * quads + k < quads_all) {
+      int4 o;
+      o.x = run;
+      o.y = o.x + q[k].x;
+      o.z = o.y + q[k].y;
+      o.w = o.z + q[k].z;
+      s4[k] = o;
+      run = o.w + q[k].w;
+    }
+  cluster.sync();
+
+  for (int p = gt; p < P.ntot; p += kNaAll) bin_key(P, p);
+  cluster.sync();
+  for (int p = gt; p < P.ntot; p += kNaAll) bin_scatter<true>(P, p, false);
 }
 
 // Device address of the scratch on each device, looked up once per device
@@ -168,14 +242,14 @@ extern "C" int dpd_forces_noalloc(int64_t n, const float *pos, const float *vel,
   P.nbox = 1;
   P.single = make_box_dev(bp, 0, 0, (int)n);
 
-  const int padded = scan_tiles((int)ncell) * kScanTile;
-  k_noalloc_reset<<<(padded + 255) / 256, 256, 0, s>>>(padded, (unsigned long long)step);
+  k_noalloc_bin<<<kNaBlocks, kNaThreads, 0, s>>>(P, pos, vel, (unsigned long long)step);
   DPD_CUDA_TRY(cudaGetLastError());
-  DPD_CUDA_TRY(launch_load(P, 0, (int)n, pos, vel, P.single.L[0], P.single.L[1], P.single.L[2], s));
-  StepConfig cfg{};
-  cfg.rows = true;
-  DPD_CUDA_TRY(launch_step(P, false, false, cfg, s));
-  DPD_CUDA_TRY(launch_gather(P, 0, 0, (int)n, nullptr, nullptr, force, s));
+  if (rows_pay(P, false)) {
+    DPD_CUDA_TRY(launch_force_rows(P, false, false, false, s, force));
+  } else {
+    DPD_CUDA_TRY(launch_force(P, StepConfig{}, s));
+    DPD_CUDA_TRY(launch_gather(P, 0, 0, (int)n, nullptr, nullptr, force, s));
+  }
 #if defined(DPD_CHECKED) && DPD_CHECKED
   // checked build: read the error word back (the normal build does not wait)
   unsigned h = 0;

@@ -413,20 +413,39 @@ def forces_noalloc(pos, vel, L, a=25.0, gamma=4.5, kT=1.0, rc=1.0, dt=0.005, see
         if not (_is_cuda_tensor(out) and out.device == dev and out.dtype == torch.float32
                 and out.is_contiguous() and tuple(out.shape) == (n, 3)):
             raise ValueError("out must be a contiguous float32 (n, 3) tensor on pos.device")
-    with torch.cuda.device(dev):
-        pp, _, kp = _vec3_arg(pos, n)
-        vv, _, kv = _vec3_arg(vel, n)
-        if out is None:
-            out = torch.empty((n, 3), dtype=torch.float32, device=dev)
-        st = stream if stream is not None else torch.cuda.current_stream(dev)
-        L3 = np.broadcast_to(np.asarray(L, dtype=np.float64), (3,))
-        box = (ctypes.c_double * 3)(*L3)
-        check(lib().dpd_forces_noalloc(n, pp, vv, box, a, gamma, kT, rc, dt, int(seed),
-                                       int(step), ctypes.c_void_p(out.data_ptr()),
-                                       _stream_ptr(st)))
-        if isinstance(st, torch.cuda.Stream):
-            # converted copies stay allocated until the enqueued work has read them
-            for t in (kp, kv):
-                if t is not pos and t is not vel:
-                    t.record_stream(st)
+    if torch.cuda.current_device() != dev.index:
+        with torch.cuda.device(dev):
+            return _forces_noalloc(torch, dev, n, pos, vel, L, a, gamma, kT, rc, dt, seed, step,
+                                   out, stream)
+    return _forces_noalloc(torch, dev, n, pos, vel, L, a, gamma, kT, rc, dt, seed, step, out,
+                           stream)
+
+
+_Box3 = ctypes.c_double * 3
+
+
+def _forces_noalloc(torch, dev, n, pos, vel, L, a, gamma, kT, rc, dt, seed, step, out, stream):
+    # Small calls are host-bound (the two launches take about 15 us on the
+    # GPU), so inputs that need no conversion are passed as they are.
+    def vec3(x):
+        if x.dtype != torch.float32 or not x.is_contiguous():
+            x = x.detach().to(torch.float32).contiguous()
+        if x.dim() != 2 or x.shape[1] != 3 or x.shape[0] != n:
+            raise ValueError("expected an n x 3 tensor")
+        return x
+
+    kp, kv = vec3(pos), vec3(vel)
+    if out is None:
+        out = torch.empty((n, 3), dtype=torch.float32, device=dev)
+    st = stream if stream is not None else torch.cuda.current_stream(dev)
+    if isinstance(L, (tuple, list)) and len(L) == 3:
+        box = _Box3(*L)
+    else:
+        box = _Box3(*np.broadcast_to(np.asarray(L, dtype=np.float64), (3,)))
+    check(lib().dpd_forces_noalloc(n, kp.data_ptr(), kv.data_ptr(), box, a, gamma, kT, rc, dt,
+                                   int(seed), int(step), out.data_ptr(), _stream_ptr(st)))
+    if isinstance(st, torch.cuda.Stream):
+        # the inputs, or their copies, stay allocated until the enqueued work has read them
+        kp.record_stream(st)
+        kv.record_stream(st)
     return out

@@ -63,6 +63,20 @@ def test_rows_fall_back_where_a_list_overflows(dpd, stencil):
     _compare(dpd, L, x, v, stencil, "plain")
 
 
+@pytest.mark.parametrize("L,n", [((3.0, 3.0, 3.0), 1), ((3.0, 4.5, 3.2), 31), ((6.0, 6.5, 7.0), 819),
+                                 ((31.0, 31.0, 34.0), 32768), ((8.0, 8.0, 8.0), 32768)])
+def test_allocation_free_forces_equal_the_direct_routine(dpd, L, n):
+    import torch
+    x, v = uniform_box_state(L, n=n, seed=n + 1)
+    box = dpd.Box(L, seed=5, variant=0)
+    box.set_state(x, v)
+    ref = box.get_forces()
+    box.close()
+    for _ in range(2):  # the second call finds the scratch as the first left it
+        f = dpd.forces_noalloc(torch.from_numpy(x).cuda(), torch.from_numpy(v).cuda(), L, seed=5)
+        assert np.array_equal(f.cpu().numpy(), ref)
+
+
 def _compare(dpd, L, x, v, stencil, kind):
     got = _run(dpd, L, x, v, stencil, kind, None)
     ref = _run(dpd, L, x, v, stencil, kind, 0)
