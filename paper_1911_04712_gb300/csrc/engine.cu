@@ -456,7 +456,7 @@ void Engine::drop_graph() {
 int Engine::free_all() {
   void *ptrs[] = {d_.pos,   d_.vel,    d_.frc,   d_.pos2,  d_.vel2,  d_.cellOf, d_.slotIn,
                   d_.keyTmp, d_.count, d_.start, d_.bsum,  d_.boxes, d_.pbase,  d_.st,
-                  d_.work,  d_.part};
+                  d_.work,  d_.part,   d_.done};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   unsigned *err = d_.err;  // the error word lives as long as the engine
@@ -832,27 +832,27 @@ int Engine::gather(int box, float *pos, float *vel, float *frc, bool device_ptr)
   if (box < 0 || box >= nbox()) return set_error(DPD_ERR_ARG, "box index out of range");
   const int n = pbase_[box + 1] - pbase_[box];
   const Packed P = packed();
-  if (n == 0 || device_ptr) {
-    if (n > 0) DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, pos, vel, frc, stream_));
+  int *done = d_.done + d_.capW;  // the gathers' counter
+  if (n == 0) {
     int rc = fetch_error();
     if (rc) return rc;
-    DPD_CUDA_TRY(cudaStreamSynchronize(stream_));
-    return DPD_OK;
+  } else if (device_ptr) {
+    DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, pos, vel, frc, stream_, done, h_err_));
+  } else {
+    float *sp = reinterpret_cast<float *>(d_.pos2), *sv = reinterpret_cast<float *>(d_.vel2);
+    const size_t bytes = (size_t)n * 3 * sizeof(float);
+    if (pos || vel) {
+      DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, pos ? sp : nullptr, vel ? sv : nullptr,
+                                 nullptr, stream_, done, h_err_));
+      if (pos) DPD_CUDA_TRY(cudaMemcpyAsync(pos, sp, bytes, cudaMemcpyDeviceToHost, stream_));
+      if (vel) DPD_CUDA_TRY(cudaMemcpyAsync(vel, sv, bytes, cudaMemcpyDeviceToHost, stream_));
+    }
+    if (frc || !(pos || vel)) {
+      DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, nullptr, nullptr, frc ? sp : nullptr,
+                                 stream_, done, h_err_));
+      if (frc) DPD_CUDA_TRY(cudaMemcpyAsync(frc, sp, bytes, cudaMemcpyDeviceToHost, stream_));
+    }
   }
-  float *sp = reinterpret_cast<float *>(d_.pos2), *sv = reinterpret_cast<float *>(d_.vel2);
-  const size_t bytes = (size_t)n * 3 * sizeof(float);
-  if (pos || vel) {
-    DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, pos ? sp : nullptr, vel ? sv : nullptr,
-                               nullptr, stream_));
-    if (pos) DPD_CUDA_TRY(cudaMemcpyAsync(pos, sp, bytes, cudaMemcpyDeviceToHost, stream_));
-    if (vel) DPD_CUDA_TRY(cudaMemcpyAsync(vel, sv, bytes, cudaMemcpyDeviceToHost, stream_));
-  }
-  if (frc) {
-    DPD_CUDA_TRY(launch_gather(P, box, pbase_[box], n, nullptr, nullptr, sp, stream_));
-    DPD_CUDA_TRY(cudaMemcpyAsync(frc, sp, bytes, cudaMemcpyDeviceToHost, stream_));
-  }
-  int rc = fetch_error();
-  if (rc) return rc;
   DPD_CUDA_TRY(cudaStreamSynchronize(stream_));
   return DPD_OK;
 }
@@ -872,14 +872,19 @@ int Engine::build_work() {
     for (int q = s0; q < s1; q += kChunk) work_.push_back(StatsWork{b, q, std::min(q + kChunk, s1), 0});
   }
   wbeg_[nb] = (int)work_.size();
-  if (work_.size() + nb > d_.capW) {  // partials of the work items, then per-box totals
+  if (work_.size() + nb > d_.capW) {
     if (d_.work) cudaFree(d_.work);
     if (d_.part) cudaFree(d_.part);
+    if (d_.done) cudaFree(d_.done);
     d_.work = nullptr;
     d_.part = nullptr;
+    d_.done = nullptr;
+    d_.capW = 0;
     const size_t cap = (work_.size() + nb) * 2;
     DPD_CUDA_TRY(cudaMalloc(&d_.work, cap * sizeof(StatsWork)));
     DPD_CUDA_TRY(cudaMalloc(&d_.part, cap * kStatsFields * sizeof(double)));
+    DPD_CUDA_TRY(cudaMalloc(&d_.done, (cap + 1) * sizeof(int)));
+    DPD_CUDA_TRY(cudaMemsetAsync(d_.done, 0, (cap + 1) * sizeof(int), stream_));
     d_.capW = cap;
   }
   if (wbeg_.size() > cap_wbeg_) {
@@ -920,22 +925,17 @@ int Engine::box_sums(std::vector<double> &sums) {
     int rc = build_work();
     if (rc) return rc;
   }
-  // partial sums per work item, then per-box totals on the device (work
-  // order), behind the partials in the same buffer; one small copy to pinned memory
+  // one kernel writes every box's totals and the error word to pinned memory
   const size_t nsum = (size_t)nb * kStatsFields;
   if (nsum > cap_hsum_) {
     if (h_sum_) cudaFreeHost(h_sum_);
     h_sum_ = nullptr;
+    cap_hsum_ = 0;
     DPD_CUDA_TRY(cudaMallocHost(&h_sum_, nsum * 2 * sizeof(double)));
     cap_hsum_ = nsum * 2;
   }
-  double *box_out = d_.part + work_.size() * kStatsFields;  // capacity: work items + boxes
-  DPD_CUDA_TRY(launch_stats(packed(), d_.work, (int)work_.size(), d_.part, stream_, d_wbeg_, nb,
-                            box_out));
-  DPD_CUDA_TRY(cudaMemcpyAsync(h_sum_, box_out, nsum * sizeof(double), cudaMemcpyDeviceToHost,
-                               stream_));
-  int rc = fetch_error();
-  if (rc) return rc;
+  DPD_CUDA_TRY(launch_stats(packed(), d_.work, (int)work_.size(), d_wbeg_, d_.part, d_.done, h_sum_,
+                            h_err_, stream_));
   DPD_CUDA_TRY(cudaStreamSynchronize(stream_));
   sums.assign(h_sum_, h_sum_ + nsum);
   return DPD_OK;

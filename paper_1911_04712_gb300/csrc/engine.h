@@ -74,6 +74,7 @@ struct DeviceArrays {
   unsigned *err = nullptr;
   StatsWork *work = nullptr;
   double *part = nullptr;
+  int *done = nullptr;  // finished blocks: per box (statistics), then one for gathers
   size_t capP = 0, capC = 0, capB = 0, capW = 0;
 };
 

@@ -208,8 +208,14 @@ __device__ __forceinline__ void pair_add(float &hi, float &lo, float bh, float b
   lo = e - (hi - s);
 }
 
-__global__ void __launch_bounds__(kStatsThreads) k_stats(Packed P, const StatsWork *__restrict__ work,
-                                                         double *__restrict__ out) {
+// The last block of a box to finish also sums the box's work items and writes
+// its totals, and the error word, to pinned host memory.  For a small box
+// that is the whole read-out in one launch: a second kernel for the totals
+// and two copies took STATS_FIGURE.
+__global__ void __launch_bounds__(kStatsThreads)
+    k_stats(Packed P, const StatsWork *__restrict__ work, const int *__restrict__ wbeg, double *out,
+            int *__restrict__ done, double *__restrict__ host_sums,
+            unsigned *__restrict__ host_err) {
   const StatsWork w = work[blockIdx.x];
   const BoxDev &B = P.boxes[w.box];
   const BoxState S = P.st[w.box];
@@ -269,37 +275,85 @@ __global__ void __launch_bounds__(kStatsThreads) k_stats(Packed P, const StatsWo
     }
     if (lane == 0) out[(size_t)blockIdx.x * kStatsFields + F] = (double)(w.end - w.begin);
   }
+  __shared__ bool last;
+  const int w0 = wbeg[w.box], w1 = wbeg[w.box + 1];
+  if (threadIdx.x == 0) {
+    __threadfence();  // this block's sums before its count
+    last = atomicAdd(done + w.box, 1) == w1 - w0 - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  // Per-box totals in a fixed order (strided sums, then a tree), so that they
+  // do not depend on the other boxes nor on which block is last.
+  __threadfence();
+  __shared__ double box[kStatsFields][kStatsThreads];
+  const int t = threadIdx.x;
+#pragma unroll
+  for (int k = 0; k < kStatsFields; ++k) {
+    double acc[2] = {0.0, 0.0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll 4
+      for (int i = w0 + t + h * kStatsThreads; i < w1; i += 2 * kStatsThreads)
+        acc[h] += __ldcg(out + (size_t)i * kStatsFields + k);
+    box[k][t] = acc[0] + acc[1];
+  }
+  __syncthreads();
+  for (int h = kStatsThreads / 2; h > 0; h >>= 1) {
+    if (t < h)
+#pragma unroll
+      for (int k = 0; k < kStatsFields; ++k) box[k][t] += box[k][t + h];
+    __syncthreads();
+  }
+  if (t < kStatsFields) host_sums[(size_t)w.box * kStatsFields + t] = box[t][0];
+  if (t == 0) {
+    done[w.box] = 0;  // for the next read-out
+    *host_err = *P.err;
+  }
 }
 
 // ----------------------------------------------------------------- gather
+// host_err (may be null): the last block to finish also writes the error word
+// to pinned host memory, in place of a copy behind the kernel.
 __global__ void k_gather(Packed P, int box, int slot0, int n, float *__restrict__ pos3,
-                         float *__restrict__ vel3, float *__restrict__ frc3) {
+                         float *__restrict__ vel3, float *__restrict__ frc3,
+                         int *__restrict__ done, unsigned *__restrict__ host_err) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const int p = slot0 + k;
-  const float4 x = P.pos[p];
-  const int id = (int)(__float_as_uint(x.w) & kIdMask);
-  if (id >= n) {
-    atomicOr(P.err, kErrNonFinite);
-    return;
+  if (k < n) {
+    const int p = slot0 + k;
+    const float4 x = P.pos[p];
+    const int id = (int)(__float_as_uint(x.w) & kIdMask);
+    if (id >= n) {
+      atomicOr(P.err, kErrNonFinite);
+    } else {
+      const float4 f = P.frc[p];
+      if (pos3) {
+        pos3[3 * id] = x.x;
+        pos3[3 * id + 1] = x.y;
+        pos3[3 * id + 2] = x.z;
+      }
+      if (vel3) {
+        const float h = P.st[box].pending ? P.boxes[box].hdt_m : 0.0f;
+        const float4 v = P.vel[p];
+        vel3[3 * id] = fmaf(h, f.x, v.x);
+        vel3[3 * id + 1] = fmaf(h, f.y, v.y);
+        vel3[3 * id + 2] = fmaf(h, f.z, v.z);
+      }
+      if (frc3) {
+        frc3[3 * id] = f.x;
+        frc3[3 * id + 1] = f.y;
+        frc3[3 * id + 2] = f.z;
+      }
+    }
   }
-  const float4 f = P.frc[p];
-  if (pos3) {
-    pos3[3 * id] = x.x;
-    pos3[3 * id + 1] = x.y;
-    pos3[3 * id + 2] = x.z;
-  }
-  if (vel3) {
-    const float h = P.st[box].pending ? P.boxes[box].hdt_m : 0.0f;
-    const float4 v = P.vel[p];
-    vel3[3 * id] = fmaf(h, f.x, v.x);
-    vel3[3 * id + 1] = fmaf(h, f.y, v.y);
-    vel3[3 * id + 2] = fmaf(h, f.z, v.z);
-  }
-  if (frc3) {
-    frc3[3 * id] = f.x;
-    frc3[3 * id + 1] = f.y;
-    frc3[3 * id + 2] = f.z;
+  if (!host_err) return;
+  __syncthreads();  // this block's error bits
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(done, 1) == (int)gridDim.x - 1) {
+      *done = 0;  // for the next read-out
+      *host_err = atomicOr(P.err, 0u);
+    }
   }
 }
 
@@ -581,45 +635,18 @@ cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream
   return cudaEventRecord(ev[5], s);
 }
 
-// Per-box totals of the work items' partial sums (work items of a box are
-// contiguous, wbeg[b] .. wbeg[b + 1]): one block per box, each thread a
-// strided sum, then a tree in a fixed order, so a box's totals do not
-// depend on the other boxes packed with it.
-constexpr int kBoxSumThreads = 512;
-__global__ void __launch_bounds__(kBoxSumThreads)
-    k_stats_boxes(const double *__restrict__ part, const int *__restrict__ wbeg,
-                  double *__restrict__ out) {
-  __shared__ double red[kStatsFields][kBoxSumThreads];
-  const int b = blockIdx.x, t = threadIdx.x;
-  double acc[kStatsFields] = {0, 0, 0, 0, 0, 0};
-#pragma unroll 4
-  for (int w = wbeg[b] + t; w < wbeg[b + 1]; w += kBoxSumThreads)
-#pragma unroll
-    for (int k = 0; k < kStatsFields; ++k) acc[k] += part[(size_t)w * kStatsFields + k];
-#pragma unroll
-  for (int k = 0; k < kStatsFields; ++k) red[k][t] = acc[k];
-  __syncthreads();
-  for (int h = kBoxSumThreads / 2; h > 0; h >>= 1) {
-    if (t < h)
-#pragma unroll
-      for (int k = 0; k < kStatsFields; ++k) red[k][t] += red[k][t + h];
-    __syncthreads();
-  }
-  if (t < kStatsFields) out[(size_t)b * kStatsFields + t] = red[t][0];
-}
-
-cudaError_t launch_stats(const Packed &P, const StatsWork *work, int nwork, double *out,
-                         cudaStream_t s, const int *wbeg, int nbox, double *box_out) {
+cudaError_t launch_stats(const Packed &P, const StatsWork *work, int nwork, const int *wbeg,
+                         double *part, int *done, double *host_sums, unsigned *host_err,
+                         cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  k_stats<<<nwork, kStatsThreads, 0, s>>>(P, work, out);
-  if (box_out && nbox > 0) k_stats_boxes<<<nbox, kBoxSumThreads, 0, s>>>(out, wbeg, box_out);
+  k_stats<<<nwork, kStatsThreads, 0, s>>>(P, work, wbeg, part, done, host_sums, host_err);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gather(const Packed &P, int box, int slot0, int n, float *pos3, float *vel3,
-                          float *frc3, cudaStream_t s) {
+                          float *frc3, cudaStream_t s, int *done, unsigned *host_err) {
   if (n <= 0) return cudaSuccess;
-  k_gather<<<blocks_for(n, 256), 256, 0, s>>>(P, box, slot0, n, pos3, vel3, frc3);
+  k_gather<<<blocks_for(n, 256), 256, 0, s>>>(P, box, slot0, n, pos3, vel3, frc3, done, host_err);
   return cudaGetLastError();
 }
 

@@ -342,16 +342,19 @@ cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream
 constexpr int kNumStages = 5;
 constexpr int kKernelsPerStep = 6;
 
-// Per-work-item FP64 partial sums for box statistics.
-// With box_out: also the per-box totals (nbox x kStatsFields, a fixed order per box).
-cudaError_t launch_stats(const Packed &P, const StatsWork *work, int nwork, double *out,
-                         cudaStream_t s, const int *wbeg = nullptr, int nbox = 0,
-                         double *box_out = nullptr);
+// Box statistics: per-work-item FP64 partial sums in `part`, then each box's
+// totals (kStatsFields each, a fixed order per box) and the error word written
+// to pinned host memory.  done: a zero per box, left zero.
+cudaError_t launch_stats(const Packed &P, const StatsWork *work, int nwork, const int *wbeg,
+                         double *part, int *done, double *host_sums, unsigned *host_err,
+                         cudaStream_t s);
 
 // Write slots [slot0, slot0 + n) to id order as n x 3 arrays (any may be null);
-// velocities are full-step (pending half kick applied).
+// velocities are full-step (pending half kick applied).  host_err: the error
+// word is written there too (pinned host memory; done: a zero, left zero).
 cudaError_t launch_gather(const Packed &P, int box, int slot0, int n, float *pos3, float *vel3,
-                          float *frc3, cudaStream_t s);
+                          float *frc3, cudaStream_t s, int *done = nullptr,
+                          unsigned *host_err = nullptr);
 
 // Served form: device-drawn initial state of a box (uniform positions,
 // Maxwellian velocities with variance vscale^2, zero mean momentum).
