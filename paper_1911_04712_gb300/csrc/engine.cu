@@ -11,7 +11,7 @@
 
 namespace dpd {
 
-// Sets up to this size replay a call's last steps from graphs (Engine::step).
+// Sets up to this size capture graphs of a call's last steps at once (Engine::step).
 constexpr int kGraphTailSlots = 131072;
 
 static thread_local std::string t_err;
@@ -733,13 +733,23 @@ int Engine::step(int64_t nsteps) {
   int rc = DPD_OK;
   for (; graph_chunk > 1 && left >= graph_chunk; left -= graph_chunk)
     if ((rc = launch_graph(&graph_, graph_chunk))) return rc;
-  // The rest: one step is a graph of its own.  Several steps are graphs of
-  // 2^k steps where the host launches kernels (about 7 us each) slower than
-  // they run: 20 steps of an L = 24 box took 769 us by direct launches, 547
-  // by graphs, and the first call, which captures them, 792 -> 590 us
-  // (N = 41,472).  At 98,304 slots 20 steps went from 1226 to 941 us; from
-  // 140,000 on the launches keep up and steps start sooner without a capture.
-  if (graph_chunk > 1 && (left == 1 || (left > 1 && ntot_ <= kGraphTailSlots && !capturing())))
+  // The rest: one step is a graph of its own, several steps are graphs of 2^k
+  // steps, since kernels launched one by one leave gaps of some 2 to 5 us: 20
+  // steps of an L = 24 box took 769 us by direct launches, 547 by graphs; 10
+  // of the L = 64 mixture 1705 and 1571; 20 of an L = 128 box 18.21 and 17.94
+  // ms.  Capturing takes about 12 us a step.  A small set saves more than that
+  // at the first call (N = 41,472: 792 -> 590 us); a larger one launches
+  // directly the first time and captures when a length comes again.
+  bool graphs = graph_chunk > 1 && left > 0;
+  if (graphs && left > 1) {
+    if (capturing()) {
+      graphs = false;
+    } else if (ntot_ > kGraphTailSlots && (left & ~tails_seen_) != 0) {
+      tails_seen_ |= left;
+      graphs = false;
+    }
+  }
+  if (graphs)
     for (int k = kTails - 1; k >= 0; --k)
       for (; left >= (int64_t)1 << k; left -= (int64_t)1 << k)
         if ((rc = launch_graph(&tail_[k], 1 << k))) return rc;
