@@ -456,7 +456,7 @@ void Engine::drop_graph() {
 int Engine::free_all() {
   void *ptrs[] = {d_.pos,   d_.vel,    d_.frc,   d_.pos2,  d_.vel2,  d_.cellOf, d_.slotIn,
                   d_.keyTmp, d_.count, d_.start, d_.bsum,  d_.boxes, d_.pbase,  d_.st,
-                  d_.work,  d_.part,   d_.done};
+                  d_.work,  d_.part};
   for (void *p : ptrs)
     if (p) cudaFree(p);
   unsigned *err = d_.err;  // the error word lives as long as the engine
@@ -885,15 +885,13 @@ int Engine::build_work() {
   if (work_.size() + nb > d_.capW) {
     if (d_.work) cudaFree(d_.work);
     if (d_.part) cudaFree(d_.part);
-    if (d_.done) cudaFree(d_.done);
     d_.work = nullptr;
     d_.part = nullptr;
-    d_.done = nullptr;
     d_.capW = 0;
     const size_t cap = (work_.size() + nb) * 2;
     DPD_CUDA_TRY(cudaMalloc(&d_.work, cap * sizeof(StatsWork)));
-    DPD_CUDA_TRY(cudaMalloc(&d_.part, cap * kStatsFields * sizeof(double)));
-    DPD_CUDA_TRY(cudaMalloc(&d_.done, (cap + 1) * sizeof(int)));
+    DPD_CUDA_TRY(cudaMalloc(&d_.part, cap * kStatsFields * sizeof(double) + (cap + 1) * sizeof(int)));
+    d_.done = reinterpret_cast<int *>(d_.part + cap * kStatsFields);  // one allocation
     DPD_CUDA_TRY(cudaMemsetAsync(d_.done, 0, (cap + 1) * sizeof(int), stream_));
     d_.capW = cap;
   }

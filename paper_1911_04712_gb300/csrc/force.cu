@@ -451,22 +451,6 @@ cudaError_t prepare_device() {
                               maxb);
 }
 
-// Whether the row-parallel kernels serve this box.  They win while the direct
-// kernels leave the GPU waiting.  Force stage, direct against row-parallel
-// (us, the stage's events):
-//   full  N = 1,536: 28.6 / 10.2; 55,296 (rho 4): 41.3 / 33.1; 65,856 (rho 3): 37.0 / 36.9;
-//         80,000 (rho 10): 89.4 / 68.4; 98,304 (rho 3): 40.4 / 49.2
-//   half  N = 1,536: 18.4 / 8.2; 55,296: 23.9 / 18.3; 98,304: 24.6 / 22.5;
-//         192,000 (rho 3): 39.3 / 37.5; 331,776 (rho 3): 52.3 / 59.4
-// and for Gaussian noise or several species the lines cross at 90,000 and
-// 98,304 (rho 3).  Above about 12 particles per cell the lists of a row
-// would often overflow (the kernels then fall back to the direct routine).
-constexpr int kRowsMaxFull = 65536, kRowsMaxHalf = 98304, kRowsMaxPerCell = 12;
-bool rows_pay(const Packed &P, bool half) {
-  return P.nbox == 1 && P.ntot <= (half ? kRowsMaxHalf : kRowsMaxFull) &&
-         (long long)P.ntot * kSlicesX <= (long long)kRowsMaxPerCell * P.ncell;
-}
-
 cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s, bool fuse) {
   const bool single = (P.nbox == 1);
   const bool half = (cfg.stencil == 1);
@@ -483,7 +467,7 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
   ForceBand whole{0, P.ntot, 0, 0};
   const ForceBand *bands = cfg.nbands > 0 ? cfg.band : &whole;
   const int nb = cfg.nbands > 0 ? cfg.nbands : 1;
-  if (cfg.rows && rows_pay(P, half))
+  if (cfg.rows && rows_pay(P, half, bands[0].gauss != 0))
     return launch_force_rows(P, half, bands[0].gauss != 0, fuse, s);
   for (int k = 0; k < nb; ++k) {
     const ForceBand &b = bands[k];

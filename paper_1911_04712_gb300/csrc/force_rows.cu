@@ -12,8 +12,8 @@
 // waiting for one load.  Here a step's chain is one row scan, about two pair
 // evaluations and one ordered sum.  Force stage at rho = 3, direct against
 // row-parallel: N = 1,536 full 28.6 -> 10.2 us, half 18.4 -> 8.2; N = 55,296
-// (rho = 4) full 41.3 -> 33.1, half 23.9 -> 18.3.  launch_force says where the
-// lines cross.
+// (rho = 4) full 41.3 -> 33.1, half 23.9 -> 18.3.  rows_pay says where the lines
+// cross.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -26,17 +26,35 @@ namespace dpd {
 
 namespace {
 
-constexpr int kRowsUnroll = 8;  // candidates loaded per iteration: a row's window at rho = 3
-constexpr int kRowsCap = 40;    // list places of one target in one row
+constexpr int kRowsUnroll = 4;  // candidates loaded per iteration
+// List places of one target in one row, and of a block's queue: at rho = 8
+// the own row holds 10 neighbours of 34, so that denser boxes need the longer
+// lists, which cost the others resident blocks.
+constexpr int kRowsCap = 24, kRowsCapDense = 40;
+constexpr int kRowsQueue = 1728, kRowsQueueDense = 2880;  // half of it for the half stencil
+// Resident blocks an SM the registers are held to.  With eight candidates an
+// iteration, the long lists and no bound (72 registers, three and five blocks)
+// an L = 24, rho = 4 box stepped in 40.0 us (full) and 22.6 (half), with these
+// in 35.9 and 21.4; an L = 12, rho = 3 box in 14.9 / 11.3 and 14.7 / 11.3.
+constexpr int kRowsBlocksFull = 4, kRowsBlocksHalf = 6;
 constexpr unsigned kAll = 0xffffffffu;
 
-template <bool HALF>
+// Which boxes (rows_pay).
+constexpr int kRowsMaxFull = 65536, kRowsMaxFullDense = 106496, kRowsMaxHalf = 262144;
+constexpr int kRowsMaxFullGeneral = 98304, kRowsMaxHalfGeneral = 524288;
+constexpr int kRowsMaxPerCell = 12;
+bool slots_per_cell_at_most(const Packed &P, int n) {
+  return (long long)P.ntot * kSlicesX <= (long long)n * P.ncell;
+}
+
+template <bool HALF, bool DENSE>
 struct RowsShared {
   static constexpr int kRows = HALF ? 5 : 9, kThreads = 32 * kRows;
-  static constexpr int kQueue = HALF ? 1536 : 2880;
+  static constexpr int kCap = DENSE ? kRowsCapDense : kRowsCap;
+  static constexpr int kQueue = (DENSE ? kRowsQueueDense : kRowsQueue) / (HALF ? 2 : 1);
   float4 own_pos[32], own_vel[32];
   union {
-    uint32_t list[kRowsCap * kThreads];  // entry k of thread t at k * kThreads + t
+    uint32_t list[kCap * kThreads];  // entry k of thread t at k * kThreads + t
     float4 res[HALF ? 1 : kQueue];       // after the lists were gathered
   };
   uint32_t queue[kQueue];                // list entries: rows in order, lanes in order
@@ -55,11 +73,12 @@ __device__ __forceinline__ void store3(float *__restrict__ out3, const float4 &p
   o[2] = f.z;
 }
 
-template <bool HALF, bool GAUSS>
-__global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
+template <bool HALF, bool GAUSS, bool DENSE>
+__global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
+                                  HALF ? kRowsBlocksHalf : kRowsBlocksFull)
     k_force_rows(Packed P, bool fuse, float *__restrict__ out3) {
-  using Sh = RowsShared<HALF>;
-  constexpr int NT = Sh::kThreads, U = kRowsUnroll, CAP = kRowsCap;
+  using Sh = RowsShared<HALF, DENSE>;
+  constexpr int NT = Sh::kThreads, U = kRowsUnroll, CAP = Sh::kCap;
   extern __shared__ float4 rows_smem[];
   Sh &W = *reinterpret_cast<Sh *>(rows_smem);
   const int tid = threadIdx.x, lane = tid & 31, row = tid >> 5;
@@ -238,21 +257,54 @@ __global__ void __launch_bounds__(RowsShared<HALF>::kThreads)
   if (out3 && alive) store3(out3, pi, P.frc[p]);  // this thread's own store
 }
 
-template <bool HALF, bool GAUSS>
+template <bool HALF, bool GAUSS, bool DENSE>
 cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
-  using Sh = RowsShared<HALF>;
-  k_force_rows<HALF, GAUSS><<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse, out3);
+  using Sh = RowsShared<HALF, DENSE>;
+  k_force_rows<HALF, GAUSS, DENSE>
+      <<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse, out3);
   return cudaGetLastError();
 }
 
 template <bool HALF, bool GAUSS>
+cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
+  return slots_per_cell_at_most(P, 7) ? launch_one<HALF, GAUSS, false>(P, fuse, s, out3)
+                                      : launch_one<HALF, GAUSS, true>(P, fuse, s, out3);
+}
+
+template <bool HALF, bool GAUSS>
 cudaError_t prepare_one() {
-  return cudaFuncSetAttribute(k_force_rows<HALF, GAUSS>,
+  cudaError_t e = cudaFuncSetAttribute(k_force_rows<HALF, GAUSS, false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(RowsShared<HALF, false>));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_force_rows<HALF, GAUSS, true>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(RowsShared<HALF>));
+                              (int)sizeof(RowsShared<HALF, true>));
 }
 
 }  // namespace
+
+// The row-parallel kernels win while the direct kernels leave the GPU waiting.
+// A step, direct against row-parallel (us):
+//   full  N = 40,960 (rho 10) 78.3 / 47.0; 65,856 (rho 3) 40.5 / 38.3; 81,000 (rho 3)
+//         43.0 / 44.1; 105,456 (rho 6) 73.0 / 65.5; 106,480 (rho 10) 103.9 / 98.3;
+//         279,936 (rho 6) 137.6 / 146.2
+//   half  N = 40,960 (rho 10) 42.5 / 28.4; 192,000 (rho 3) 46.6 / 41.3; 255,552 (rho 3)
+//         52.6 / 51.2; 331,776 (rho 3) 62.0 / 63.9; 552,960 (rho 5) 117.1 / 120.9
+// and the general kernels (Gaussian noise)
+//   full  N = 40,960 (rho 10) 103.0 / 50.5; 98,304 (rho 3) 55.0 / 51.1; 116,346 (rho 3,
+//         uneven edges) 62.2 / 63.9; 331,776 (rho 3) 126.8 / 137.5
+//   half  N = 255,552 (rho 3) 64.2 / 54.2; 526,848 (rho 3) 106.0 / 99.2; 2,654,208 (rho 3)
+//         478.7 / 494.0.
+// Above about 12 particles per cell the lists overflow too often.
+bool rows_pay(const Packed &P, bool half, bool general) {
+  int most = kRowsMaxHalf;
+  if (general)
+    most = half ? kRowsMaxHalfGeneral : kRowsMaxFullGeneral;
+  else if (!half)
+    most = slots_per_cell_at_most(P, 5) ? kRowsMaxFull : kRowsMaxFullDense;
+  return P.nbox == 1 && P.ntot <= most && slots_per_cell_at_most(P, kRowsMaxPerCell);
+}
 
 cudaError_t prepare_rows() {
   cudaError_t e = prepare_one<false, false>();

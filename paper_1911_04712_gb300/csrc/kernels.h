@@ -143,7 +143,7 @@ cudaError_t prepare_rows();
 // out3: also write the forces to id order (n x 3, full stencil).
 cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s,
                               float *out3 = nullptr);
-bool rows_pay(const Packed &P, bool half);  // whether they serve this box
+bool rows_pay(const Packed &P, bool half, bool general);  // whether they serve this box
 
 // Direct force-kernel variants (threads per block, pair-list capacity).
 int force_variant_info(int v, int *threads, int *cap);

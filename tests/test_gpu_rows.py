@@ -44,7 +44,8 @@ def _run(dpd, L, x, v, stencil, kind, variant):
 
 CASES = [((3.0, 3.0, 3.0), 1), ((3.0, 3.0, 3.0), 31), ((3.0, 3.4, 3.9), 33),
          ((5.0, 6.5, 7.25), 707), ((40.0, 3.0, 3.5), 97), ((8.0, 8.0, 8.0), 6144),
-         ((26.0, 26.0, 26.0), 65536), ((26.0, 26.0, 26.0), 65537)]
+         ((26.0, 26.0, 26.0), 65536), ((26.0, 26.0, 26.0), 65537),
+         ((8.0, 9.0, 10.0), 5041), ((8.0, 9.0, 10.0), 8640)]  # long lists; 12 per cell
 
 
 @pytest.mark.parametrize("stencil", [0, 1])
