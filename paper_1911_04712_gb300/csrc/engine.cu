@@ -231,8 +231,8 @@ int Engine::build_bands() {
     if (v == kBrickVariant && 30.0 * B.np / ((double)B.n[0] * B.n[1] * B.n[2]) >
                                   0.5 * kBrickCaps)
       v = 0;
-    const int g = B.noise != 0 || B.nspec > 1;  // general kernel
-    if (!runs.empty() && runs.back().variant == v && runs.back().gauss == g) {
+    const int g = (B.noise != 0 ? 1 : 0) | (B.nspec > 1 ? 2 : 0);  // general kernel
+    if (!runs.empty() && runs.back().variant == v && runs.back().gen == g) {
       runs.back().slot1 = pbase_[b + 1];
       runs.back().item1 = brick_beg_[b + 1];
       runs.back().box1 = b + 1;
@@ -249,10 +249,10 @@ int Engine::build_bands() {
     // too fragmented (boxes not ordered by band): one launch with the
     // variant that covers the most particles
     std::vector<long long> cover(kNumForceVariants, 0);
-    int anyg = 0;
+    int anyg = runs[0].gen;
     for (const auto &r : runs) {
       cover[r.variant] += r.slot1 - r.slot0;
-      anyg |= r.gauss;
+      if (r.gen != anyg) anyg = 3;  // the kernel that looks at each box
     }
     const int best = (int)(std::max_element(cover.begin(), cover.end()) - cover.begin());
     runs.assign(1, ForceBand{0, ntot_, best, anyg});
@@ -608,7 +608,7 @@ int Engine::update_params(const std::vector<BoxParams> &params) {
   drop_graph();
   DPD_CUDA_TRY(cudaMemcpyAsync(d_.boxes, boxes_.data(), boxes_.size() * sizeof(BoxDev),
                                cudaMemcpyHostToDevice, stream_));
-  return DPD_OK;
+  return build_bands();  // the noise decides on the force kernel
 }
 
 int Engine::load_box(int box, const float *pos, const float *vel, bool device_ptr,

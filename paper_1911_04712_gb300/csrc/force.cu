@@ -4,7 +4,7 @@
 // them; the variants differ in block size, list capacity and how a warp
 // drains its lists (per lane, balanced in list order, or spread over the
 // lanes with atomic sums), chosen per density band from tuning tables.
-// General variants also serve Gaussian noise and several species.  The full
+// General variants serve Gaussian noise, several species, or both.  The full
 // stencil can fuse the next step's integrate into its epilogue.  Plus the
 // optional shared-memory staged tiles.
 #include <cuda_runtime.h>
@@ -24,9 +24,11 @@ constexpr int kTileListCap = 24;
 
 static inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 
-// One thread per target slot in [slot0, slot1).
-template <bool SINGLE, bool HALF, int NT, int CAP, bool BAL, bool GAUSS, bool SPREAD>
-__global__ void __launch_bounds__(NT) k_force(Packed P, int slot0, int slot1, bool fuse) {
+// One thread per target slot in [slot0, slot1).  The full stencil's Gaussian
+// kernel is held to the registers of seven blocks an SM: its math functions
+// let it grow to 80, and a step of an L = 64, rho = 3 box to 256 us (243 so).
+template <bool SINGLE, bool HALF, int NT, int CAP, bool BAL, int GEN, bool SPREAD>
+__global__ void __launch_bounds__(NT, (GEN == kGenGauss && !HALF) ? 7 : 0) k_force(Packed P, int slot0, int slot1, bool fuse) {
   constexpr int kListWords = BAL ? 1 : CAP * NT;
   __shared__ uint32_t smem_list[kListWords];
   __shared__ WarpScratch<BAL ? CAP : 4> smem_warp[BAL ? NT / 32 : 1];
@@ -50,15 +52,15 @@ __global__ void __launch_bounds__(NT) k_force(Packed P, int slot0, int slot1, bo
   auto run = [&](const BoxDev &B) {
     if constexpr (BAL) {
       WarpScratch<CAP> *W = &smem_warp[threadIdx.x >> 5];
-      force_direct<HALF, NT, CAP, true, GAUSS>(P, B, S, p, alive,
+      force_direct<HALF, NT, CAP, true, GEN>(P, B, S, p, alive,
                                                W->list + (threadIdx.x & 31) * (CAP + 1), W,
                                                nullptr, mixed, fuse, real);
     } else if constexpr (SPREAD) {
-      force_direct<HALF, NT, CAP, false, GAUSS, true>(P, B, S, p, alive, smem_list + threadIdx.x,
+      force_direct<HALF, NT, CAP, false, GEN, true>(P, B, S, p, alive, smem_list + threadIdx.x,
                                                       nullptr, smem_own + (threadIdx.x >> 5) * 64,
                                                       mixed, fuse, real);
     } else {
-      force_direct<HALF, NT, CAP, false, GAUSS>(P, B, S, p, alive, smem_list + threadIdx.x,
+      force_direct<HALF, NT, CAP, false, GEN>(P, B, S, p, alive, smem_list + threadIdx.x,
                                                 nullptr, nullptr, false, fuse, real);
     }
   };
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(NT) k_force(Packed P, int slot0, int slot1, bo
 // The warps of a packed set whose slots span two boxes, one block of 32
 // threads each (first slots in warp_start), with the per-lane drain: each
 // lane evaluates only its own pairs, with its own box's parameters.
-template <bool HALF, int CAP, bool GAUSS>
+template <bool HALF, int CAP, int GEN>
 __global__ void __launch_bounds__(32)
     k_force_warps(Packed P, const int *__restrict__ warp_start, int slot1, bool fuse) {
   __shared__ uint32_t smem_list[CAP * 32];
@@ -81,7 +83,7 @@ __global__ void __launch_bounds__(32)
   const int b = find_box(P.pbase, P.nbox, min(p, P.ntot - 1));
   const BoxState S = P.st[b];
   const bool alive = real && S.adv;
-  force_direct<HALF, 32, CAP, false, GAUSS>(P, P.boxes[b], S, p, alive, smem_list + threadIdx.x,
+  force_direct<HALF, 32, CAP, false, GEN>(P, P.boxes[b], S, p, alive, smem_list + threadIdx.x,
                                             nullptr, nullptr, false, fuse, real);
 }
 
@@ -398,23 +400,31 @@ int force_variant_info(int v, int *threads, int *cap) {
   return 0;
 }
 
-template <bool SINGLE, bool HALF, int NT, int CAP, bool BAL = false, bool GAUSS = false,
+template <bool SINGLE, bool HALF, int NT, int CAP, bool BAL = false, int GEN = 0,
           bool SPREAD = false>
 static void launch_k(const Packed &P, int s0, int s1, bool fuse, cudaStream_t s) {
   if (s1 > s0)
-    k_force<SINGLE, HALF, NT, CAP, BAL, GAUSS, SPREAD && HALF>
+    k_force<SINGLE, HALF, NT, CAP, BAL, GEN, SPREAD && HALF>
         <<<blocks_for(s1 - s0, NT), NT, 0, s>>>(P, s0, s1, fuse);
 }
 
+// The general kernels: spread drain for the half stencil, else per lane.  One
+// for each of Gaussian noise and several species beside the one for both: the
+// half stencil's need 56 registers where that needs 78, and a step of an L =
+// 64, rho = 3 box takes 127.6 and 124.8 us in place of 147.5 and 144.9.
+template <bool SINGLE, bool HALF, int GEN>
+static void launch_general(const Packed &P, int s0, int s1, bool fuse, cudaStream_t s) {
+  launch_k<SINGLE, HALF, 128, 24, false, GEN, HALF>(P, s0, s1, fuse, s);
+}
+
 template <bool SINGLE, bool HALF>
-static void launch_variant(int v, bool gauss, const Packed &P, int s0, int s1, bool fuse,
+static void launch_variant(int v, int gen, const Packed &P, int s0, int s1, bool fuse,
                            cudaStream_t s) {
-  if (gauss) {  // general kernels: bands holding Gaussian-noise or several-species boxes
-    if constexpr (HALF)
-      launch_k<SINGLE, HALF, 128, 24, false, true, true>(P, s0, s1, fuse, s);  // spread drain
-    else
-      launch_k<SINGLE, HALF, 128, 24, false, true>(P, s0, s1, fuse, s);
-    return;
+  switch (gen) {  // bands of Gaussian-noise or several-species boxes
+    case 0: break;
+    case kGenGauss: return launch_general<SINGLE, HALF, kGenGauss>(P, s0, s1, fuse, s);
+    case kGenSpecies: return launch_general<SINGLE, HALF, kGenSpecies>(P, s0, s1, fuse, s);
+    default: return launch_general<SINGLE, HALF, kGenGauss | kGenSpecies>(P, s0, s1, fuse, s);
   }
   switch (v) {
     case 1: launch_k<SINGLE, HALF, 128, 16>(P, s0, s1, fuse, s); break;
@@ -426,9 +436,9 @@ static void launch_variant(int v, bool gauss, const Packed &P, int s0, int s1, b
     case 7: launch_k<SINGLE, HALF, 64, 24, true>(P, s0, s1, fuse, s); break;
     case 8: launch_k<SINGLE, HALF, 128, 24, true>(P, s0, s1, fuse, s); break;
     case 9: launch_k<SINGLE, HALF, 256, 24, true>(P, s0, s1, fuse, s); break;
-    case 10: launch_k<SINGLE, HALF, 64, 32, false, false, true>(P, s0, s1, fuse, s); break;
-    case 11: launch_k<SINGLE, HALF, 128, 32, false, false, true>(P, s0, s1, fuse, s); break;
-    case 12: launch_k<SINGLE, HALF, 128, 24, false, false, true>(P, s0, s1, fuse, s); break;
+    case 10: launch_k<SINGLE, HALF, 64, 32, false, 0, true>(P, s0, s1, fuse, s); break;
+    case 11: launch_k<SINGLE, HALF, 128, 32, false, 0, true>(P, s0, s1, fuse, s); break;
+    case 12: launch_k<SINGLE, HALF, 128, 24, false, 0, true>(P, s0, s1, fuse, s); break;
     default: launch_k<SINGLE, HALF, 128, 24>(P, s0, s1, fuse, s); break;
   }
 }
@@ -467,17 +477,17 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
   ForceBand whole{0, P.ntot, 0, 0};
   const ForceBand *bands = cfg.nbands > 0 ? cfg.band : &whole;
   const int nb = cfg.nbands > 0 ? cfg.nbands : 1;
-  if (cfg.rows && rows_pay(P, half, bands[0].gauss != 0))
-    return launch_force_rows(P, half, bands[0].gauss != 0, fuse, s);
+  if (cfg.rows && rows_pay(P, half, bands[0].gen != 0))
+    return launch_force_rows(P, half, bands[0].gen, fuse, s);
   for (int k = 0; k < nb; ++k) {
     const ForceBand &b = bands[k];
-    if (half && !b.gauss && b.variant == kBrickVariant && cfg.nbands > 0 && cfg.bricks.items) {
+    if (half && !b.gen && b.variant == kBrickVariant && cfg.nbands > 0 && cfg.bricks.items) {
       const cudaError_t e = launch_force_brick(P, cfg.bricks, b.item0, b.item1, s);
       if (e != cudaSuccess) return e;
       continue;
     }
     if (!single && cfg.grouped && cfg.hboxes && cfg.nbands > 0 &&
-        grouped_variant(b.variant, b.gauss != 0, half)) {
+        grouped_variant(b.variant, b.gen != 0, half)) {
       // box-grouped launches: no warp spans two boxes
       const cudaError_t e = launch_force_group(P, cfg.hboxes, b.box0, b.box1, b.variant, s);
       if (e != cudaSuccess) return e;
@@ -485,25 +495,25 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
     }
     if (single) {
       if (half)
-        launch_variant<true, true>(b.variant, b.gauss, P, b.slot0, b.slot1, false, s);
+        launch_variant<true, true>(b.variant, b.gen, P, b.slot0, b.slot1, false, s);
       else
-        launch_variant<true, false>(b.variant, b.gauss, P, b.slot0, b.slot1, fuse, s);
+        launch_variant<true, false>(b.variant, b.gen, P, b.slot0, b.slot1, fuse, s);
     } else {
       if (half)
-        launch_variant<false, true>(b.variant, b.gauss, P, b.slot0, b.slot1, false, s);
+        launch_variant<false, true>(b.variant, b.gen, P, b.slot0, b.slot1, false, s);
       else
-        launch_variant<false, false>(b.variant, b.gauss, P, b.slot0, b.slot1, fuse, s);
+        launch_variant<false, false>(b.variant, b.gen, P, b.slot0, b.slot1, fuse, s);
       // the band's two-box warps, skipped by the warp-cooperative kernels
       if (cfg.nbands > 0 && b.mw_count > 0 && cfg.mixed_warps &&
-          cooperative_variant(b.variant, b.gauss != 0, half)) {
+          cooperative_variant(b.variant, b.gen != 0, half)) {
         const int *ws = cfg.mixed_warps + b.mw_off;
         if (half) {
-          if (b.gauss)
-            k_force_warps<true, 24, true><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, false);
+          if (b.gen)
+            k_force_warps<true, 24, kGenGauss | kGenSpecies><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, false);
           else
-            k_force_warps<true, 24, false><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, false);
+            k_force_warps<true, 24, 0><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, false);
         } else {
-          k_force_warps<false, 24, false><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, fuse);
+          k_force_warps<false, 24, 0><<<b.mw_count, 32, 0, s>>>(P, ws, b.slot1, fuse);
         }
       }
     }

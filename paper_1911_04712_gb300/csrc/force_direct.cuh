@@ -16,6 +16,9 @@ namespace dpd {
 // Candidates loaded per iteration of the candidate pass.
 constexpr int kScanUnroll = 4;
 
+// What the general kernels serve (GEN): Gaussian noise, several species, both.
+constexpr int kGenGauss = 1, kGenSpecies = 2;
+
 // ------------------------------------------------------------------ force
 // Pair lists: each thread appends the neighbours found inside rc to its own
 // column of a shared-memory list (entry k of thread t at lst[k * NT + t], NT threads),
@@ -91,7 +94,10 @@ __device__ __forceinline__ void pair_vector(const BX &B, uint32_t e, const float
 
 // Force of the pair at r_ij = (dx, dy, dz), 0 < r2 = r_ij^2 < rc^2, on i (3),
 // and r . F^C.  wi, wj: the particles' id words; (slo, shi): the noise step.
-template <bool GAUSS, typename BX>
+// GEN: what the box may have beyond uniform noise and one species (kGenGauss,
+// kGenSpecies); a kernel for one of them takes it for granted, the kernel for
+// both looks at the box.  All give the same bits for the same box.
+template <int GEN, typename BX>
 __device__ __forceinline__ float4 pair_force(const BX &B, float dx, float dy, float dz, float r2,
                                              const float4 &ui, const float4 &vj, uint32_t wi,
                                              uint32_t wj, uint32_t slo, uint32_t shi) {
@@ -99,15 +105,15 @@ __device__ __forceinline__ float4 pair_force(const BX &B, float dx, float dy, fl
   // several species, whose pair of species picks them (and a cut-off
   // rc_st <= rc that the pair must be inside)
   float pa = B.a, pgam = B.gamma, psig = B.sig, psig_g = 0.f, pinv_rc = B.inv_rc;
-  if constexpr (GAUSS) {
-    psig_g = B.sig_g;
-    if (B.nspec > 1) {
+  if constexpr (GEN & kGenGauss) psig_g = B.sig_g;
+  if constexpr (GEN & kGenSpecies) {
+    if (GEN == kGenSpecies || B.nspec > 1) {
       const int k = (int)((wi >> kSpeciesShift) * kMaxSpecies + (wj >> kSpeciesShift));
       if (!(r2 < B.sp_rc2[k])) return make_float4(0.f, 0.f, 0.f, 0.f);
       pa = B.sp_a[k];
       pgam = B.sp_gamma[k];
       psig = B.sp_sig[k];
-      psig_g = B.sp_sig_g[k];
+      if constexpr (GEN & kGenGauss) psig_g = B.sp_sig_g[k];
       pinv_rc = B.sp_inv_rc[k];
     }
     wi &= kIdMask;  // the pair noise takes the ids alone
@@ -118,19 +124,22 @@ __device__ __forceinline__ float4 pair_force(const BX &B, float dx, float dy, fl
   const float w = fmaxf(fmaf(-r, pinv_rc, 1.0f), 0.0f);
   const float wR = B.kexp == 1.0f ? w : powf(w, B.kexp);
   const float ev = fmaf(dx, ui.x - vj.x, fmaf(dy, ui.y - vj.y, dz * (ui.z - vj.z))) * rinv;
-  float fr;  // random term sigma w_R xi / sqrt(dt)
-  if constexpr (GAUSS) {  // general kernels: Gaussian noise or several species
+  float amp, xi;  // random term sigma w_R xi / sqrt(dt)
+  if constexpr (GEN & kGenGauss) {
     const uint2 u = pair_words(wi, wj, slo, shi, B.seed_lo, B.seed_hi);
-    if (B.noise == 0)
-      fr = psig * wR * noise_int(u.x);
-    else
-      fr = psig_g * wR * gauss_xi(u.x, u.y);
+    if (GEN == kGenGauss || B.noise != 0) {
+      amp = psig_g * wR;
+      xi = gauss_xi(u.x, u.y);
+    } else {
+      amp = psig * wR;
+      xi = noise_int(u.x);
+    }
   } else {
-    const uint32_t u = pair_word(wi, wj, slo, shi, B.seed_lo, B.seed_hi);
-    fr = psig * wR * noise_int(u);
+    amp = psig * wR;
+    xi = noise_int(pair_word(wi, wj, slo, shi, B.seed_lo, B.seed_hi));
   }
   const float fc = pa * w;
-  const float s = (fr + fmaf(-pgam * wR * wR, ev, fc)) * rinv;
+  const float s = fmaf(amp, xi, fmaf(-pgam * wR * wR, ev, fc)) * rinv;
   // rounded products (no fusion into the caller's sums), so that every
   // drain order-preserving variant adds exactly the same terms
   return make_float4(__fmul_rn(s, dx), __fmul_rn(s, dy), __fmul_rn(s, dz), __fmul_rn(fc, r));
@@ -198,7 +207,7 @@ __device__ __forceinline__ void finish_force(const Packed &P, const BX &B, const
 // lane holds more than FLUSH entries.  BX is the type holding the box
 // constants: BoxDev, or the compact BoxHot of a grouped launch (uniform
 // noise, one species, half stencil).
-template <bool HALF, int NT, int CAP, bool BAL = false, bool GAUSS = false, bool SPREAD = false,
+template <bool HALF, int NT, int CAP, bool BAL = false, int GEN = 0, bool SPREAD = false,
           typename BX = BoxDev>
 __device__ __forceinline__ void force_direct(const Packed &P, const BX &B, const BoxState &S,
                                              int p, bool alive, uint32_t *__restrict__ lst,
@@ -247,7 +256,7 @@ __device__ __forceinline__ void force_direct(const Packed &P, const BX &B, const
     float dx, dy, dz;
     pair_vector(B, e, qi, pj, dx, dy, dz);
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float4 g = pair_force<GAUSS>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
+    const float4 g = pair_force<GEN>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
                                        __float_as_uint(pj.w), slo, shi);
     if constexpr (HALF) atomicAdd(P.frc + j, make_float4(-g.x, -g.y, -g.z, g.w));
     return g;

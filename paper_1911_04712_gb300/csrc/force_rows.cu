@@ -40,8 +40,9 @@ constexpr int kRowsBlocksFull = 4, kRowsBlocksHalf = 6;
 constexpr unsigned kAll = 0xffffffffu;
 
 // Which boxes (rows_pay).
-constexpr int kRowsMaxFull = 65536, kRowsMaxFullDense = 106496, kRowsMaxHalf = 262144;
-constexpr int kRowsMaxFullGeneral = 98304, kRowsMaxHalfGeneral = 524288;
+constexpr int kRowsMaxHalf = 262144;
+constexpr int kRowsMaxFull = 65536, kRowsMaxFullDense = 106496;  // dense: above 5 per cell
+constexpr int kRowsMaxFullGeneral = 90112, kRowsMaxFullGeneralDense = 139264;
 constexpr int kRowsMaxPerCell = 12;
 bool slots_per_cell_at_most(const Packed &P, int n) {
   return (long long)P.ntot * kSlicesX <= (long long)n * P.ncell;
@@ -73,7 +74,7 @@ __device__ __forceinline__ void store3(float *__restrict__ out3, const float4 &p
   o[2] = f.z;
 }
 
-template <bool HALF, bool GAUSS, bool DENSE>
+template <bool HALF, int GEN, bool DENSE>
 __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
                                   HALF ? kRowsBlocksHalf : kRowsBlocksFull)
     k_force_rows(Packed P, bool fuse, float *__restrict__ out3) {
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
   if (W.overflow || total > Sh::kQueue) {
     // a denser place than the lists hold: the direct routine, by one warp
     if (row == 0) {
-      force_direct<HALF, NT, CAP, false, GAUSS>(P, P.single, S, p, alive, W.list + tid, nullptr,
+      force_direct<HALF, NT, CAP, false, GEN>(P, P.single, S, p, alive, W.list + tid, nullptr,
                                                 nullptr, false, fuse, real);
       if (out3 && alive) store3(out3, pi, P.frc[p]);
     }
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
     float dx, dy, dz;
     pair_vector(B, e, qi, pj, dx, dy, dz);
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-    const float4 g = pair_force<GAUSS>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
+    const float4 g = pair_force<GEN>(B, dx, dy, dz, r2, ui, vj, __float_as_uint(qi.w),
                                        __float_as_uint(pj.w), (uint32_t)S.step,
                                        (uint32_t)(S.step >> 32));
     if constexpr (HALF) {
@@ -257,27 +258,27 @@ __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
   if (out3 && alive) store3(out3, pi, P.frc[p]);  // this thread's own store
 }
 
-template <bool HALF, bool GAUSS, bool DENSE>
+template <bool HALF, int GEN, bool DENSE>
 cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
   using Sh = RowsShared<HALF, DENSE>;
-  k_force_rows<HALF, GAUSS, DENSE>
+  k_force_rows<HALF, GEN, DENSE>
       <<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse, out3);
   return cudaGetLastError();
 }
 
-template <bool HALF, bool GAUSS>
+template <bool HALF, int GEN>
 cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
-  return slots_per_cell_at_most(P, 7) ? launch_one<HALF, GAUSS, false>(P, fuse, s, out3)
-                                      : launch_one<HALF, GAUSS, true>(P, fuse, s, out3);
+  return slots_per_cell_at_most(P, 7) ? launch_one<HALF, GEN, false>(P, fuse, s, out3)
+                                      : launch_one<HALF, GEN, true>(P, fuse, s, out3);
 }
 
-template <bool HALF, bool GAUSS>
+template <bool HALF, int GEN>
 cudaError_t prepare_one() {
-  cudaError_t e = cudaFuncSetAttribute(k_force_rows<HALF, GAUSS, false>,
+  cudaError_t e = cudaFuncSetAttribute(k_force_rows<HALF, GEN, false>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)sizeof(RowsShared<HALF, false>));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_force_rows<HALF, GAUSS, true>,
+  return cudaFuncSetAttribute(k_force_rows<HALF, GEN, true>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)sizeof(RowsShared<HALF, true>));
 }
@@ -291,37 +292,45 @@ cudaError_t prepare_one() {
 //         279,936 (rho 6) 137.6 / 146.2
 //   half  N = 40,960 (rho 10) 42.5 / 28.4; 192,000 (rho 3) 46.6 / 41.3; 255,552 (rho 3)
 //         52.6 / 51.2; 331,776 (rho 3) 62.0 / 63.9; 552,960 (rho 5) 117.1 / 120.9
-// and the general kernels (Gaussian noise)
-//   full  N = 40,960 (rho 10) 103.0 / 50.5; 98,304 (rho 3) 55.0 / 51.1; 116,346 (rho 3,
-//         uneven edges) 62.2 / 63.9; 331,776 (rho 3) 126.8 / 137.5
-//   half  N = 255,552 (rho 3) 64.2 / 54.2; 526,848 (rho 3) 106.0 / 99.2; 2,654,208 (rho 3)
-//         478.7 / 494.0.
+// and the general kernels (Gaussian noise; several species)
+//   full  N = 65,856 (rho 3) 46.1 / 38.9; 42.6 / 38.5, 98,304 (rho 3) 55.2 / 50.2; 49.1 /
+//         49.8, 116,346 (rho 3, uneven edges) 57.5 / 63.9, 138,240 (rho 10) 167.6 / 128.0;
+//         140.6 / 124.9
+//   half  N = 255,552 (rho 3) 55.5 / 53.1; 54.6 / 52.0, 331,776 (rho 3) 66.4 / 66.5; 64.6 / 65.1.
 // Above about 12 particles per cell the lists overflow too often.
 bool rows_pay(const Packed &P, bool half, bool general) {
+  const bool dense = !slots_per_cell_at_most(P, 5);
   int most = kRowsMaxHalf;
-  if (general)
-    most = half ? kRowsMaxHalfGeneral : kRowsMaxFullGeneral;
+  if (!half && general)
+    most = dense ? kRowsMaxFullGeneralDense : kRowsMaxFullGeneral;
   else if (!half)
-    most = slots_per_cell_at_most(P, 5) ? kRowsMaxFull : kRowsMaxFullDense;
+    most = dense ? kRowsMaxFullDense : kRowsMaxFull;
   return P.nbox == 1 && P.ntot <= most && slots_per_cell_at_most(P, kRowsMaxPerCell);
 }
 
 cudaError_t prepare_rows() {
-  cudaError_t e = prepare_one<false, false>();
-  if (e == cudaSuccess) e = prepare_one<false, true>();
-  if (e == cudaSuccess) e = prepare_one<true, false>();
-  if (e == cudaSuccess) e = prepare_one<true, true>();
+  cudaError_t e = cudaSuccess;
+  for (cudaError_t (*one)() :
+       {prepare_one<false, 0>, prepare_one<false, 1>, prepare_one<false, 2>, prepare_one<false, 3>,
+        prepare_one<true, 0>, prepare_one<true, 1>, prepare_one<true, 2>, prepare_one<true, 3>})
+    if (e == cudaSuccess) e = one();
   return e;
 }
 
-cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s,
+template <bool HALF>
+static cudaError_t launch_gen(const Packed &P, int gen, bool fuse, cudaStream_t s, float *out3) {
+  switch (gen) {
+    case 0: return launch_one<HALF, 0>(P, fuse, s, out3);
+    case kGenGauss: return launch_one<HALF, kGenGauss>(P, fuse, s, out3);
+    case kGenSpecies: return launch_one<HALF, kGenSpecies>(P, fuse, s, out3);
+    default: return launch_one<HALF, kGenGauss | kGenSpecies>(P, fuse, s, out3);
+  }
+}
+
+cudaError_t launch_force_rows(const Packed &P, bool half, int gen, bool fuse, cudaStream_t s,
                               float *out3) {
   if (P.nbox != 1 || (half && (fuse || out3))) return cudaErrorInvalidValue;
-  if (half)
-    return general ? launch_one<true, true>(P, fuse, s, out3)
-                   : launch_one<true, false>(P, fuse, s, out3);
-  return general ? launch_one<false, true>(P, fuse, s, out3)
-                 : launch_one<false, false>(P, fuse, s, out3);
+  return half ? launch_gen<true>(P, gen, fuse, s, out3) : launch_gen<false>(P, gen, fuse, s, out3);
 }
 
 }  // namespace dpd

@@ -65,7 +65,7 @@ cudaError_t launch_force_brick(const Packed &P, const BrickGrid &G, int i0, int 
 // A contiguous slot range whose force kernel uses one variant.
 struct ForceBand {
   int slot0, slot1, variant;
-  int gauss;  // 1: the band needs the general kernel (Gaussian noise or several species)
+  int gen;    // the general kernel it needs, if any: 1 Gaussian noise, 2 several species, 3 both
   // packed sets: the band's warps whose slots span two boxes (first slots at
   // StepConfig::mixed_warps[mw_off ..]); warp-cooperative variants skip them
   // and a second launch runs them with the per-lane drain
@@ -141,7 +141,7 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
 // Row-parallel force kernels of one small box (force_rows.cu).
 cudaError_t prepare_rows();
 // out3: also write the forces to id order (n x 3, full stencil).
-cudaError_t launch_force_rows(const Packed &P, bool half, bool general, bool fuse, cudaStream_t s,
+cudaError_t launch_force_rows(const Packed &P, bool half, int gen, bool fuse, cudaStream_t s,
                               float *out3 = nullptr);
 bool rows_pay(const Packed &P, bool half, bool general);  // whether they serve this box
 

@@ -90,3 +90,24 @@ def _compare(dpd, L, x, v, stencil, kind):
         # three steps later the states differ by the rounding of the sums
         assert np.abs(got[1].astype(np.float64) - ref[1]).max() <= 10 * FORCE_TOL * rms
         assert np.abs(got[2].astype(np.float64) - ref[2]).max() <= 3 * 0.005 * FORCE_TOL * rms
+
+
+@pytest.mark.parametrize("n", [700, 131000])
+@pytest.mark.parametrize("stencil", [0, 1])
+def test_noise_changed_on_a_loaded_box(dpd, n, stencil):
+    """The force kernel follows the noise: a box whose noise is changed after
+    loading steps as one that had it from the start."""
+    L = 6.0 if n < 1000 else 36.0
+    x, v = uniform_box_state(L, n=n, seed=2)
+    for before, after in ((0, 1), (1, 0)):
+        out = []
+        for first in (before, after):
+            box = dpd.Box(L, seed=8, stencil=stencil, noise=first)
+            box.set_state(x, v)
+            box.set_param(dpd.PARAM_NOISE, after)
+            box.set_state(x, v)
+            out.append(box.get_forces())
+            box.close()
+        rms = float(np.sqrt((out[1].astype(np.float64) ** 2).sum(1).mean()))
+        err = np.abs(out[0].astype(np.float64) - out[1]).max()
+        assert err <= (0.0 if stencil == 0 else FORCE_TOL * rms)
