@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
   const int p0 = (int)blockIdx.x * 32, p = p0 + lane;
   const bool real = p < P.ntot;
   const BoxDev &B = P.single;
+  step_begin();
   const BoxState S = P.st[0];
   const bool alive = real && S.adv && DPD_IN_BOUNDS(p >= 0 && p < P.ntot, P.err);
   float4 pi = make_float4(0.f, 0.f, 0.f, 0.f), vi = pi;
@@ -261,9 +262,8 @@ __global__ void __launch_bounds__(RowsShared<HALF, DENSE>::kThreads,
 template <bool HALF, int GEN, bool DENSE>
 cudaError_t launch_one(const Packed &P, bool fuse, cudaStream_t s, float *out3) {
   using Sh = RowsShared<HALF, DENSE>;
-  k_force_rows<HALF, GEN, DENSE>
-      <<<(P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s>>>(P, fuse, out3);
-  return cudaGetLastError();
+  return launch_step_kernel(P.ntot <= kEarlySlots, k_force_rows<HALF, GEN, DENSE>,
+                            (P.ntot + 31) / 32, Sh::kThreads, sizeof(Sh), s, P, fuse, out3);
 }
 
 template <bool HALF, int GEN>

@@ -45,6 +45,7 @@ __global__ void k_load(Packed P, int slot0, int n, const float *__restrict__ pos
 // ------------------------------------------------------- integrate + count
 template <bool SINGLE>
 __global__ void __launch_bounds__(kBinThreads) k_integrate_bin(Packed P, bool move) {
+  step_begin();
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
   int b = 0;
   if constexpr (!SINGLE) b = find_box_warp(P.pbase, P.nbox, min(p, P.ntot - 1));
@@ -90,6 +91,7 @@ __device__ __forceinline__ int block_excl_scan(int v, int *total) {
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int *__restrict__ count,
                                                               int *__restrict__ bsum) {
+  step_begin();
   const int4 *c4 = reinterpret_cast<const int4 *>(count) +
                    (size_t)blockIdx.x * (kScanTile / 4) + threadIdx.x * (kScanItems / 4);
   int s = 0;
@@ -124,6 +126,7 @@ __global__ void __launch_bounds__(1024) k_scan_bsum(int *__restrict__ bsum, int 
 // its own; otherwise it holds their exclusive scan.
 __global__ void __launch_bounds__(kScanThreads)
     k_scan_apply(Packed P, bool advance, bool sum_tiles) {
+  step_begin();
   int4 *c4 = reinterpret_cast<int4 *>(P.count) + (size_t)blockIdx.x * (kScanTile / 4) +
              threadIdx.x * (kScanItems / 4);
   int4 *s4 = reinterpret_cast<int4 *>(P.start) + (size_t)blockIdx.x * (kScanTile / 4) +
@@ -183,12 +186,14 @@ __global__ void __launch_bounds__(kScanThreads)
 // ---------------------------------------------------------------- reorder
 __global__ void __launch_bounds__(kBinThreads) k_bin_keys(Packed P) {
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
+  step_begin();
   if (p < P.ntot) bin_key(P, p);
 }
 
 template <bool STABLE>
 __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(Packed P, bool zero_frc) {
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
+  step_begin();
   if (p < P.ntot) bin_scatter<STABLE>(P, p, zero_frc);
 }
 
@@ -577,32 +582,47 @@ cudaError_t launch_load(const Packed &P, int slot0, int n, const float *pos3, co
 // (event times, with the gaps between launches).  Beyond that the sums are
 // scanned by one block.
 constexpr int kScanSumTiles = 2048;
-static void launch_scan(const Packed &P, bool advance, cudaStream_t s) {
+static void launch_scan(const Packed &P, bool advance, bool early, cudaStream_t s) {
   const int nt = scan_tiles(P.ncell);
-  if (nt > 1) k_scan_reduce<<<nt, kScanThreads, 0, s>>>(P.count, P.bsum);
+  if (nt > 1) launch_step_kernel(early, k_scan_reduce, nt, kScanThreads, 0, s, P.count, P.bsum);
   if (nt > kScanSumTiles) k_scan_bsum<<<1, 1024, 0, s>>>(P.bsum, nt);
-  k_scan_apply<<<nt, kScanThreads, 0, s>>>(P, advance, nt <= kScanSumTiles);
+  launch_step_kernel(early, k_scan_apply, nt, kScanThreads, 0, s, P, advance,
+                     nt <= kScanSumTiles);
+}
+
+static void launch_integrate(const Packed &P, bool move, bool early, cudaStream_t s) {
+  const int gb = blocks_for(P.ntot, kBinThreads);
+  if (P.nbox == 1)
+    launch_step_kernel(early, k_integrate_bin<true>, gb, kBinThreads, 0, s, P, move);
+  else
+    launch_step_kernel(early, k_integrate_bin<false>, gb, kBinThreads, 0, s, P, move);
+}
+
+// The full stencil's key pass.
+static void launch_keys(const Packed &P, bool early, cudaStream_t s) {
+  launch_step_kernel(early, k_bin_keys, blocks_for(P.ntot, kBinThreads), kBinThreads, 0, s, P);
+}
+
+// half: by arrival rank, clearing the forces for the half stencil's sums.
+static void launch_scatter(const Packed &P, bool half, bool early, cudaStream_t s) {
+  const int gb = blocks_for(P.ntot, kBinThreads);
+  if (half)
+    launch_step_kernel(early, k_bin_scatter<false>, gb, kBinThreads, 0, s, P, true);
+  else
+    launch_step_kernel(early, k_bin_scatter<true>, gb, kBinThreads, 0, s, P, false);
 }
 
 cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConfig &cfg,
                         cudaStream_t s, bool fused_in, bool fuse_out) {
   if (P.ntot <= 0) return cudaSuccess;
-  const bool single = (P.nbox == 1);
-  const int gb = blocks_for(P.ntot, kBinThreads);
-  if (fused_in) {
-    // row a1 of this step ran in the previous step's force kernel
-  } else if (single) {
-    k_integrate_bin<true><<<gb, kBinThreads, 0, s>>>(P, move);
-  } else {
-    k_integrate_bin<false><<<gb, kBinThreads, 0, s>>>(P, move);
-  }
-  launch_scan(P, advance, s);
-  if (cfg.stencil == 1) {
-    k_bin_scatter<false><<<gb, kBinThreads, 0, s>>>(P, true);
-  } else {
-    k_bin_keys<<<gb, kBinThreads, 0, s>>>(P);
-    k_bin_scatter<true><<<gb, kBinThreads, 0, s>>>(P, false);
-  }
+  const bool half = cfg.stencil == 1;
+  const bool early = cfg.rows && P.ntot <= kEarlySlots &&
+                     rows_pay(P, half, cfg.nbands > 0 && cfg.band[0].gen != 0);
+  // fused_in: row a1 of this step ran in the previous step's force kernel
+  if (!fused_in) launch_integrate(P, move, early, s);
+  launch_scan(P, advance, early, s);
+  if (!half) launch_keys(P, early, s);
+  launch_scatter(P, half, early, s);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_force(P, cfg, s, fuse_out && cfg.stencil == 0);
@@ -611,23 +631,16 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
 cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,
                               cudaEvent_t *ev) {
   if (P.ntot <= 0) return cudaSuccess;
-  const bool single = (P.nbox == 1);
-  const int gb = blocks_for(P.ntot, kBinThreads);
+  const bool half = cfg.stencil == 1;
   cudaError_t e;
   if ((e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  if (single)
-    k_integrate_bin<true><<<gb, kBinThreads, 0, s>>>(P, true);
-  else
-    k_integrate_bin<false><<<gb, kBinThreads, 0, s>>>(P, true);
+  launch_integrate(P, true, false, s);
   if ((e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
-  launch_scan(P, true, s);
+  launch_scan(P, true, false, s);
   if ((e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
-  if (cfg.stencil != 1) k_bin_keys<<<gb, kBinThreads, 0, s>>>(P);
+  if (!half) launch_keys(P, false, s);
   if ((e = cudaEventRecord(ev[3], s)) != cudaSuccess) return e;
-  if (cfg.stencil == 1)
-    k_bin_scatter<false><<<gb, kBinThreads, 0, s>>>(P, true);
-  else
-    k_bin_scatter<true><<<gb, kBinThreads, 0, s>>>(P, false);
+  launch_scatter(P, half, false, s);
   if ((e = cudaEventRecord(ev[4], s)) != cudaSuccess) return e;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_force(P, cfg, s)) != cudaSuccess) return e;
