@@ -670,13 +670,16 @@ int Engine::capture_graph(int nsteps, cudaGraphExec_t *out) {
     cudaGraphExecDestroy(*out);
     *out = nullptr;
   }
-  const Packed P = packed();
+  Packed P = packed();
   cudaGraph_t g = nullptr;
   DPD_CUDA_TRY(cudaStreamBeginCapture(cap_, cudaStreamCaptureModeThreadLocal));
   cudaError_t e = cudaSuccess;
   const bool fz = fused_steps();  // steps inside the chunk fused, the last one plain
+  const bool swap = swap_pays(P, cfg_);  // pairs of steps exchange the arrays and exchange them back
   for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-    e = launch_step(P, true, true, cfg_, cap_, fz && k > 0, fz && k + 1 < nsteps);
+    e = swap && (k | 1) < nsteps
+            ? launch_step_swapped(P, cfg_, cap_)
+            : launch_step(P, true, true, cfg_, cap_, fz && k > 0, fz && k + 1 < nsteps);
     if (e == cudaSuccess && sample_every_ > 0)
       e = launch_sample(P, d_.work, (int)work_.size(), d_wbeg_, d_from_, sample_every_, nbins_,
                         d_spart_, d_acc_, cap_);
@@ -753,10 +756,14 @@ int Engine::step(int64_t nsteps) {
     for (int k = kTails - 1; k >= 0; --k)
       for (; left >= (int64_t)1 << k; left -= (int64_t)1 << k)
         if ((rc = launch_graph(&tail_[k], 1 << k))) return rc;
-  const Packed P = packed();
+  Packed P = packed();
+  const bool swap = swap_pays(P, cfg_);
   const bool fz = fused_steps();  // the last step of the call stays plain: read-outs follow
   for (int64_t k = 0; k < left; ++k) {
-    DPD_CUDA_TRY(launch_step(P, true, true, cfg_, stream_, fz && k > 0, fz && k + 1 < left));
+    if (swap && (k | 1) < left)
+      DPD_CUDA_TRY(launch_step_swapped(P, cfg_, stream_));
+    else
+      DPD_CUDA_TRY(launch_step(P, true, true, cfg_, stream_, fz && k > 0, fz && k + 1 < left));
     int rc = launch_extra(P, stream_);
     if (rc) return rc;
   }

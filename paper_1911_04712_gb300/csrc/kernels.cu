@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <utility>
 
 #include "dpd_device.cuh"
 #include "kernels.h"
@@ -56,6 +57,41 @@ __global__ void __launch_bounds__(kBinThreads) k_integrate_bin(Packed P, bool mo
   // a stopped box (a step with nothing left to take) keeps its slots and forces
   integrate_one(P, B, p, P.pos[p], P.vel[p], f.x, f.y, f.z, mv, P.st[b].pending != 0,
                 move && !mv);
+}
+
+// Row a1 of the half stencil's larger sets, split so that the reorder finishes
+// it: this kernel kicks the velocities and clears the forces where they are,
+// and counts the cells of the new positions without storing these; the
+// reorder (k_drift_scatter) drifts the old position again with the stored
+// velocity, the same operations and so the same bits, and writes to the other
+// pair of position and velocity arrays.  Both kernels are bound by HBM: a
+// step moves 152 B a particle (48 + 36 here, 36 + 32 there) in place of the 176
+// of k_integrate_bin and k_bin_scatter.
+template <bool SINGLE>
+__global__ void __launch_bounds__(kBinThreads) k_kick_bin(Packed P) {
+  const int p = blockIdx.x * kBinThreads + threadIdx.x;
+  int b = 0;
+  if constexpr (!SINGLE) b = find_box_warp(P.pbase, P.nbox, min(p, P.ntot - 1));
+  if (p >= P.ntot) return;
+  const BoxDev B = box_of<SINGLE>(P, b);
+  const bool mv = P.st[b].remaining > 0;  // a stopped box keeps its slots and forces
+  float4 x = P.pos[p], v = P.vel[p];
+  if (mv) {
+    const float4 f = P.frc[p];
+    kick(B, v, f.x, f.y, f.z, P.st[b].pending != 0);
+    drift(P, B, x, v);
+  }
+  const int cx = cell_axis(x.x, B.invh[0], B.n[0]);
+  const int cy = cell_axis(x.y, B.invh[1], B.n[1]);
+  const int cz = cell_axis(x.z, B.invh[2], B.n[2]);
+  const int c = B.cellBase + (cz * B.n[1] + cy) * B.n[0] + cx;
+  if (mv) {
+    v.w = __int_as_float(pack_cell(cx, cy, cz));
+    P.vel[p] = v;
+    P.frc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
+  P.slotIn[p] = atomicAdd(P.count + c, 1);
 }
 
 // ------------------------------------------------------------------ scan
@@ -195,6 +231,31 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_scatter(Packed P, bool zero
   const int p = blockIdx.x * kBinThreads + threadIdx.x;
   step_begin();
   if (p < P.ntot) bin_scatter<STABLE>(P, p, zero_frc);
+}
+
+// The reorder after k_kick_bin, by arrival rank, into pos2 and vel2.
+template <bool SINGLE>
+__global__ void __launch_bounds__(kBinThreads) k_drift_scatter(Packed P) {
+  const int p = blockIdx.x * kBinThreads + threadIdx.x;
+  int b = 0;
+  if constexpr (!SINGLE) b = find_box_warp(P.pbase, P.nbox, min(p, P.ntot - 1));
+  if (p >= P.ntot) return;
+  const BoxDev B = box_of<SINGLE>(P, b);
+  const bool moved = P.st[b].adv != 0;
+  float4 x = P.pos[p];
+  const float4 v = P.vel[p];
+  int dst = p;
+  if (moved) {
+    int cx, cy, cz;
+    unpack_cell(__float_as_int(v.w), cx, cy, cz);
+    const int c = B.cellBase + (cz * B.n[1] + cy) * B.n[0] + cx;
+    if (!DPD_IN_BOUNDS(c >= 0 && c < P.ncell, P.err)) return;
+    dst = P.start[c] + P.slotIn[p];
+    if (!DPD_IN_BOUNDS(dst >= 0 && dst < P.start[c + 1] && dst < P.ntot, P.err)) return;
+    drift(P, B, x, v);
+  }
+  P.pos2[dst] = x;
+  P.vel2[dst] = v;
 }
 
 // ------------------------------------------------------------------ stats
@@ -626,6 +687,28 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_force(P, cfg, s, fuse_out && cfg.stencil == 0);
+}
+
+bool swap_pays(const Packed &P, const StepConfig &cfg) {
+  return cfg.stencil == 1 && P.ntot > kSwapSlots;
+}
+
+cudaError_t launch_step_swapped(Packed &P, const StepConfig &cfg, cudaStream_t s) {
+  if (P.ntot <= 0) return cudaSuccess;
+  const int gb = blocks_for(P.ntot, kBinThreads);
+  if (P.nbox == 1)
+    k_kick_bin<true><<<gb, kBinThreads, 0, s>>>(P);
+  else
+    k_kick_bin<false><<<gb, kBinThreads, 0, s>>>(P);
+  launch_scan(P, true, false, s);
+  if (P.nbox == 1)
+    k_drift_scatter<true><<<gb, kBinThreads, 0, s>>>(P);
+  else
+    k_drift_scatter<false><<<gb, kBinThreads, 0, s>>>(P);
+  std::swap(P.pos, P.pos2);
+  std::swap(P.vel, P.vel2);
+  cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_force(P, cfg, s);
 }
 
 cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,

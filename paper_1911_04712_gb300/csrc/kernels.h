@@ -12,7 +12,8 @@ namespace dpd {
 // single-box kernels read box constants from the parameter bank.
 struct Packed {
   float4 *pos, *vel, *frc;     // primary arrays, cell order
-  float4 *pos2, *vel2;         // integrated copies before the reorder; staging
+  float4 *pos2, *vel2;         // integrated copies before the reorder, or the other pair of
+                               // a step that exchanges them; staging
   int *cellOf;                 // packed global cell of each slot (pre-reorder order)
   int *slotIn;                 // arrival rank of each slot inside its cell
   int *keyTmp;                 // old slot index at each arrival position
@@ -198,6 +199,45 @@ __device__ __forceinline__ float refold(float x, float L) {
 // are (the half stencil's reorder otherwise clears the forces).
 constexpr int kKeepSlot = (int)0x80000000u;
 
+// The kicks of row a1: the second half kick of the previous step (when
+// `pending`), then the first of this step.
+template <typename BX>
+__device__ __forceinline__ void kick(const BX &B, float4 &v, float fx, float fy, float fz,
+                                     bool pending) {
+  const float h = B.hdt_m;
+  if (pending) {
+    v.x = fmaf(h, fx, v.x);
+    v.y = fmaf(h, fy, v.y);
+    v.z = fmaf(h, fz, v.z);
+  }
+  v.x = fmaf(h, fx, v.x);
+  v.y = fmaf(h, fy, v.y);
+  v.z = fmaf(h, fz, v.z);
+}
+
+// The drift of row a1 and the periodic wrap.
+template <typename BX>
+__device__ __forceinline__ void drift(const Packed &P, const BX &B, float4 &x, const float4 &v) {
+  x.x = wrap_coord(fmaf(B.dt, v.x, x.x), B.L[0]);
+  x.y = wrap_coord(fmaf(B.dt, v.y, x.y), B.L[1]);
+  x.z = wrap_coord(fmaf(B.dt, v.z, x.z), B.L[2]);
+  const bool finite = isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
+                      isfinite(v.y) && isfinite(v.z);
+  if (!finite) {
+    atomicOr(P.err, kErrNonFinite);
+    x.x = isfinite(x.x) ? x.x : 0.0f;
+    x.y = isfinite(x.y) ? x.y : 0.0f;
+    x.z = isfinite(x.z) ? x.z : 0.0f;
+  }
+  if (!(x.x >= 0.0f && x.x < B.L[0] && x.y >= 0.0f && x.y < B.L[1] && x.z >= 0.0f &&
+        x.z < B.L[2])) {
+    atomicOr(P.err, kErrRunaway);  // moved more than one edge in a step
+    x.x = refold(x.x, B.L[0]);
+    x.y = refold(x.y, B.L[1]);
+    x.z = refold(x.z, B.L[2]);
+  }
+}
+
 // Row a1 for the particle in slot p (Sec. 3.1 item 5, Eq. 1; Sec. 3.2): if
 // `move`, the second half kick of the previous step (when `pending`), this
 // step's first half kick with the force (fx, fy, fz), the drift and the
@@ -211,33 +251,8 @@ __device__ __forceinline__ void integrate_one(const Packed &P, const BX &B, int 
                                               float4 v, float fx, float fy, float fz, bool move,
                                               bool pending, bool keep = false) {
   if (move) {
-    const float h = B.hdt_m;
-    if (pending) {  // second half kick of the previous step
-      v.x = fmaf(h, fx, v.x);
-      v.y = fmaf(h, fy, v.y);
-      v.z = fmaf(h, fz, v.z);
-    }
-    v.x = fmaf(h, fx, v.x);  // first half kick of this step
-    v.y = fmaf(h, fy, v.y);
-    v.z = fmaf(h, fz, v.z);
-    x.x = wrap_coord(fmaf(B.dt, v.x, x.x), B.L[0]);
-    x.y = wrap_coord(fmaf(B.dt, v.y, x.y), B.L[1]);
-    x.z = wrap_coord(fmaf(B.dt, v.z, x.z), B.L[2]);
-    const bool finite = isfinite(x.x) && isfinite(x.y) && isfinite(x.z) && isfinite(v.x) &&
-                        isfinite(v.y) && isfinite(v.z);
-    if (!finite) {
-      atomicOr(P.err, kErrNonFinite);
-      x.x = isfinite(x.x) ? x.x : 0.0f;
-      x.y = isfinite(x.y) ? x.y : 0.0f;
-      x.z = isfinite(x.z) ? x.z : 0.0f;
-    }
-    if (!(x.x >= 0.0f && x.x < B.L[0] && x.y >= 0.0f && x.y < B.L[1] && x.z >= 0.0f &&
-          x.z < B.L[2])) {
-      atomicOr(P.err, kErrRunaway);  // moved more than one edge in a step
-      x.x = refold(x.x, B.L[0]);
-      x.y = refold(x.y, B.L[1]);
-      x.z = refold(x.z, B.L[2]);
-    }
+    kick(B, v, fx, fy, fz, pending);
+    drift(P, B, x, v);
   }
   const int cx = cell_axis(x.x, B.invh[0], B.n[0]);
   const int cy = cell_axis(x.y, B.invh[1], B.n[1]);
@@ -368,6 +383,16 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
 // One step with events recorded around its stages: ev[0] before the
 // integrate/count kernel, then after it, after the scan, after the key pass,
 // after the reorder and after the force kernel (6 events).
+// A half-stencil step that moves less (k_kick_bin): the state goes from pos and
+// vel to pos2 and vel2, which are exchanged in P.  Steps come in pairs, so that
+// a call leaves the state where it found it.  A step of an L = 128 box went from
+// 854 to 831 us, L = 96 375 to 366, L = 64 118.4 to 116.1 (rho = 8: 541 to 533),
+// of 512 packed boxes 1842 to 1821, of an L = 29 box (73,167 slots) 23.2 to
+// 23.0.  Below kSwapSlots small boxes launch their kernels early instead, and
+// their arrays are in L2, where the bytes hardly count.
+cudaError_t launch_step_swapped(Packed &P, const StepConfig &cfg, cudaStream_t s);
+bool swap_pays(const Packed &P, const StepConfig &cfg);
+constexpr int kSwapSlots = 65536;
 cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,
                               cudaEvent_t *ev);
 constexpr int kNumStages = 5;
