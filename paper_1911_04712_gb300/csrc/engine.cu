@@ -682,7 +682,7 @@ int Engine::capture_graph(int nsteps, cudaGraphExec_t *out) {
             : launch_step(P, true, true, cfg_, cap_, fz && k > 0, fz && k + 1 < nsteps);
     if (e == cudaSuccess && sample_every_ > 0)
       e = launch_sample(P, d_.work, (int)work_.size(), d_wbeg_, d_from_, sample_every_, nbins_,
-                        d_spart_, d_acc_, cap_);
+                        d_spart_, d_acc_, d_.done, cap_);
   }
   cudaError_t e2 = cudaStreamEndCapture(cap_, &g);
   if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -998,7 +998,7 @@ int Engine::ensure_sampling_buffers() {
 int Engine::launch_extra(const Packed &P, cudaStream_t s) {
   if (sample_every_ <= 0) return DPD_OK;
   DPD_CUDA_TRY(launch_sample(P, d_.work, (int)work_.size(), d_wbeg_, d_from_, sample_every_,
-                             nbins_, d_spart_, d_acc_, s));
+                             nbins_, d_spart_, d_acc_, d_.done, s));
   return DPD_OK;
 }
 

@@ -542,10 +542,15 @@ __global__ void k_repack(const float4 *__restrict__ opos, const float4 *__restri
 // Statistics sample of every box whose step is a multiple of `every` and
 // past its window start: per work item FP64 partials of sum v^2, sum r.F^C
 // (frc.w, each pair counted twice) and per-slab sums of the flow-axis
-// velocity with their counts.
-__global__ void __launch_bounds__(256) k_sample(Packed P, const StatsWork *__restrict__ work,
-                                                const long long *__restrict__ from, int every,
-                                                int nbins, double *__restrict__ part) {
+// velocity with their counts.  The last block of a box to finish adds the
+// box's partials (in work order) to its accumulators: acc[b] = {samples,
+// sum v^2, sum frc.w, slab sums[nbins], slab counts[nbins]}.  It runs behind
+// every step, so its cost on the steps that no box samples is its launch: a
+// second kernel for the accumulators took 3.2 us a step.
+__global__ void __launch_bounds__(256)
+    k_sample(Packed P, const StatsWork *__restrict__ work, const int *__restrict__ wbeg,
+             const long long *__restrict__ from, int every, int nbins, double *__restrict__ part,
+             double *__restrict__ acc, int *__restrict__ done) {
   extern __shared__ double sbin[];  // 2 * nbins: sums then counts
   const StatsWork w = work[blockIdx.x];
   const BoxState S = P.st[w.box];
@@ -553,10 +558,7 @@ __global__ void __launch_bounds__(256) k_sample(Packed P, const StatsWork *__res
   double *out = part + (size_t)blockIdx.x * fields;
   const bool take = S.adv && every > 0 && (long long)S.step > from[w.box] &&
                     (S.step % (unsigned long long)every) == 0ull;
-  if (!take) {
-    if (threadIdx.x == 0) out[0] = 0.0;  // marks "no sample"
-    return;
-  }
+  if (!take) return;  // the same for all blocks of a box
   for (int k = threadIdx.x; k < 2 * nbins; k += blockDim.x) sbin[k] = 0.0;
   __syncthreads();
   const BoxDev B = P.boxes[w.box];
@@ -599,30 +601,28 @@ __global__ void __launch_bounds__(256) k_sample(Packed P, const StatsWork *__res
       a += red[0][q];
       c += red[1][q];
     }
-    out[0] = 1.0;
     out[1] = a;
     out[2] = c;
   }
   for (int k = threadIdx.x; k < 2 * nbins; k += blockDim.x) out[3 + k] = sbin[k];
-}
-
-// Add each box's work-item partials (in work order) to its accumulators:
-// acc[b] = {samples, sum v^2, sum frc.w, slab sums[nbins], slab counts[nbins]}.
-__global__ void k_sample_acc(const StatsWork *__restrict__ work, const int *__restrict__ wbeg,
-                             int nbox, int nbins, const double *__restrict__ part,
-                             double *__restrict__ acc) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nbox) return;
-  const int fields = 3 + 2 * nbins;
-  const int w0 = wbeg[b], w1 = wbeg[b + 1];
-  if (w1 <= w0 || part[(size_t)w0 * fields] == 0.0) return;
-  double *a = acc + (size_t)b * fields;
-  a[0] += 1.0;
-  for (int k = 1; k < fields; ++k) {
+  __shared__ bool last;
+  __threadfence();  // this block's partials before its count
+  __syncthreads();
+  const int w0 = wbeg[w.box], w1 = wbeg[w.box + 1];
+  if (threadIdx.x == 0) last = atomicAdd(done + w.box, 1) == w1 - w0 - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double *a = acc + (size_t)w.box * fields;
+  for (int k = threadIdx.x; k < fields; k += blockDim.x) {
     double s = 0.0;
-    for (int w = w0; w < w1; ++w) s += part[(size_t)w * fields + k];
+    if (k == 0)
+      s = 1.0;
+    else
+      for (int i = w0; i < w1; ++i) s += __ldcg(part + (size_t)i * fields + k);
     a[k] += s;
   }
+  if (threadIdx.x == 0) done[w.box] = 0;  // for the next sample or read-out
 }
 
 // ================================================================ launchers
@@ -779,10 +779,10 @@ cudaError_t launch_repack(const float4 *opos, const float4 *ovel, float4 *npos, 
 
 cudaError_t launch_sample(const Packed &P, const StatsWork *work, int nwork, const int *wbeg,
                           const long long *from, int every, int nbins, double *part, double *acc,
-                          cudaStream_t s) {
+                          int *done, cudaStream_t s) {
   if (nwork <= 0 || every <= 0) return cudaSuccess;
-  k_sample<<<nwork, 256, 2 * nbins * sizeof(double), s>>>(P, work, from, every, nbins, part);
-  k_sample_acc<<<blocks_for(P.nbox, 128), 128, 0, s>>>(work, wbeg, P.nbox, nbins, part, acc);
+  k_sample<<<nwork, 256, 2 * nbins * sizeof(double), s>>>(P, work, wbeg, from, every, nbins, part,
+                                                          acc, done);
   return cudaGetLastError();
 }
 

@@ -422,7 +422,7 @@ cudaError_t launch_repack(const float4 *opos, const float4 *ovel, float4 *npos, 
 // Statistics sample (boxes whose step is a multiple of `every` past from[b]).
 cudaError_t launch_sample(const Packed &P, const StatsWork *work, int nwork, const int *wbeg,
                           const long long *from, int every, int nbins, double *part, double *acc,
-                          cudaStream_t s);
+                          int *done, cudaStream_t s);
 
 cudaError_t launch_debug_rng(const uint32_t *lo, const uint32_t *hi, long long n, uint64_t step,
                              uint64_t seed, int noise, uint32_t *out, uint32_t *out1, float *xi,
