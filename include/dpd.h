@@ -112,8 +112,8 @@ typedef struct dpd_ctx dpd_ctx;
                                      kick, drift and bin every particle for the next step of the
                                      same dpd_step call (no separate integrate pass, no stored
                                      force in between); 0 runs them as separate kernels.  Both
-                                     give the same bits.  Off for the half stencil, the staged
-                                     tiles and steps followed by sampling. */
+                                     give the same bits.  Off for the half stencil and the
+                                     staged tiles. */
 
 #define DPD_NOISE_UNIFORM 0   /* xi = sqrt(3)(2U - 1): uniform, unit variance, bit-exact on CPU */
 #define DPD_NOISE_GAUSSIAN 1  /* xi Gaussian as Sec. 2.1 states: Box-Muller on words 0 and 1,

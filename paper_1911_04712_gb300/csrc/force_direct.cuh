@@ -189,10 +189,12 @@ __device__ __forceinline__ void finish_force(const Packed &P, const BX &B, const
   } else if (fuse) {
     // the full stencil's force on p is complete here: the next step's row a1
     // for p, instead of storing the force for a separate integrate pass.  A
-    // box that stops after this step keeps its force for later read-outs.
+    // box that stops after this step keeps its force for later read-outs; under
+    // sampling every box does (its positions and velocities of this step stay in
+    // pos and vel until the next reorder).
     const bool moves = S.remaining > 0;
     integrate_one(P, B, p, pi, vi, fx, fy, fz, moves, true, !moves);
-    if (!moves) P.frc[p] = make_float4(fx, fy, fz, vir);
+    if (!moves || P.keep_frc) P.frc[p] = make_float4(fx, fy, fz, vir);
   } else {
     P.frc[p] = make_float4(fx, fy, fz, vir);
   }

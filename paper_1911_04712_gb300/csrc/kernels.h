@@ -25,6 +25,7 @@ struct Packed {
   BoxState *st;
   unsigned *err;
   int ntot, ncell, nbox;
+  int keep_frc;                // a fused step stores its forces too (a sampling pass reads them)
   BoxDev single;
 };
 
