@@ -738,7 +738,10 @@ int Engine::step(int64_t nsteps) {
   }
   int64_t left = nsteps;
   int rc = DPD_OK;
-  for (; graph_chunk > 1 && left >= graph_chunk; left -= graph_chunk)
+  // A stream that the caller is capturing takes plain launches, which become
+  // nodes of the caller's graph: no graph may be instantiated meanwhile.
+  bool graphs = graph_chunk > 1 && !capturing();
+  for (; graphs && left >= graph_chunk; left -= graph_chunk)
     if ((rc = launch_graph(&graph_, graph_chunk))) return rc;
   // The rest: one step is a graph of its own, several steps are graphs of 2^k
   // steps, since kernels launched one by one leave gaps of some 2 to 5 us: 20
@@ -747,14 +750,9 @@ int Engine::step(int64_t nsteps) {
   // ms.  Capturing takes about 12 us a step.  A small set saves more than that
   // at the first call (N = 41,472: 792 -> 590 us); a larger one launches
   // directly the first time and captures when a length comes again.
-  bool graphs = graph_chunk > 1 && left > 0;
-  if (graphs && left > 1) {
-    if (capturing()) {
-      graphs = false;
-    } else if (ntot_ > kGraphTailSlots && (left & ~tails_seen_) != 0) {
-      tails_seen_ |= left;
-      graphs = false;
-    }
+  if (graphs && left > 1 && ntot_ > kGraphTailSlots && (left & ~tails_seen_) != 0) {
+    tails_seen_ |= left;
+    graphs = false;
   }
   if (graphs)
     for (int k = kTails - 1; k >= 0; --k)
