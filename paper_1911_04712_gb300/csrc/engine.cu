@@ -11,9 +11,6 @@
 
 namespace dpd {
 
-// Sets up to this size capture graphs of a call's last steps at once (Engine::step).
-constexpr int kGraphTailSlots = 131072;
-
 static thread_local std::string t_err;
 
 int set_error(int code, const char *fmt, ...) {
@@ -748,13 +745,16 @@ int Engine::step(int64_t nsteps) {
   for (; graphs && left >= graph_chunk; left -= graph_chunk)
     if ((rc = launch_graph(&graph_, graph_chunk))) return rc;
   // The rest: one step is a graph of its own, several steps are graphs of 2^k
-  // steps, since kernels launched one by one leave gaps of some 2 to 5 us: 20
-  // steps of an L = 24 box took 769 us by direct launches, 547 by graphs; 10
-  // of the L = 64 mixture 1705 and 1571; 20 of an L = 128 box 18.21 and 17.94
-  // ms.  Capturing takes about 12 us a step.  A small set saves more than that
-  // at the first call (N = 41,472: 792 -> 590 us); a larger one launches
-  // directly the first time and captures when a length comes again.
-  if (graphs && left > 1 && ntot_ > kGraphTailSlots && (left & ~tails_seen_) != 0) {
+  // steps, since kernels launched one by one leave gaps: 20 steps of an L = 24,
+  // rho = 4 box (half stencil) take 500 us so, of the L = 64 mixture 10 take 1571
+  // and 1705 directly, of an L = 128 box 20 take 17.94 and 18.21 ms.  Capturing
+  // takes about 12 us a step before the GPU starts, so a number of steps is
+  // launched directly until it comes again: the first call of 20 steps on a new
+  // box took (full / half stencil) 680 / 524 us captured and 492 / 338 launched
+  // for N = 20,000, 1027 / 683 and 834 / 498 for 65,000, 1389 / 879 and 1419 / 854
+  // for 131,000; of 2 steps 121 / 104 and 75 / 69, 157 / 120 and 110 / 76, 203 /
+  // 144 and 176 / 114.
+  if (graphs && left > 1 && (left & ~tails_seen_) != 0) {
     tails_seen_ |= left;
     graphs = false;
   }

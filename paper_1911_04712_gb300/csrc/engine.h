@@ -232,7 +232,7 @@ class Engine {
   // 2^k steps: what a call leaves after its whole chunks
   static constexpr int kTails = 5;
   cudaGraphExec_t tail_[kTails] = {};
-  int64_t tails_seen_ = 0;  // the lengths 2^k that larger sets have run before
+  int64_t tails_seen_ = 0;  // the lengths 2^k that have run since the graphs were dropped
   int launch_graph(cudaGraphExec_t *g, int nsteps);
   bool capturing() const;  // the caller's stream is being captured
 };

@@ -1,7 +1,7 @@
 """Which calls of several steps make graphs of the engine's own.  Graphs cost
-their capture, so a large set launches directly until a number of steps comes
-again, and starts anew when its graphs were dropped (a changed parameter, a
-new layout).
+their capture, so a set launches directly until a number of steps comes again,
+and starts anew when its graphs were dropped (a changed parameter, a new
+layout).
 
 To see it, the calls run while another stream of this thread is being captured:
 CUDA refuses to instantiate a graph then, so that a call that wants a new one
@@ -45,8 +45,8 @@ def _box(dpd, n, stencil):
 
 
 @pytest.mark.parametrize("stencil", [0, 1])
-def test_large_sets_capture_when_a_length_comes_again(dpd, stencil):
-    n = 131200
+@pytest.mark.parametrize("n", [131200, 700, 66000])
+def test_sets_capture_when_a_length_comes_again(dpd, n, stencil):
     box, L = _box(dpd, n, stencil)
     _step_without_new_graphs(box, 5)
     for change in (lambda: box.set_param(dpd.PARAM_BODYFORCE, 0.1),
