@@ -231,8 +231,16 @@ int Engine::build_bands() {
     if (v == kBrickVariant && 30.0 * B.np / ((double)B.n[0] * B.n[1] * B.n[2]) >
                                   0.5 * kBrickCaps)
       v = 0;
-    const int g = (B.noise != 0 ? 1 : 0) | (B.nspec > 1 ? 2 : 0);  // general kernel
-    if (!runs.empty() && runs.back().variant == v && runs.back().gen == g) {
+    // Neighbours that need a general kernel share a band, which takes the kernel
+    // of their kind if they are of one, else the kernel that looks at each box.
+    // A launch for each kind costs more than its kernel gains: 16 Gaussian and 16
+    // two-species boxes of 1,500 particles stepped in 79 us (full stencil) and 92
+    // (half) apart, in 50 and 57 together; of 6,000 particles in 102 and 100, 97
+    // and 79; only of 20,000 in 257 and 141, 269 and 152.  Four of each in turn
+    // took 254 us apart, 44 together.
+    const int g = (B.noise != 0 ? 1 : 0) | (B.nspec > 1 ? 2 : 0);
+    if (!runs.empty() && runs.back().variant == v && (runs.back().gen != 0) == (g != 0)) {
+      if (runs.back().gen != g) runs.back().gen = 3;
       runs.back().slot1 = pbase_[b + 1];
       runs.back().item1 = brick_beg_[b + 1];
       runs.back().box1 = b + 1;
