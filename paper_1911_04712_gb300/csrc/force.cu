@@ -477,7 +477,7 @@ cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
   ForceBand whole{0, P.ntot, 0, 0};
   const ForceBand *bands = cfg.nbands > 0 ? cfg.band : &whole;
   const int nb = cfg.nbands > 0 ? cfg.nbands : 1;
-  if (cfg.rows && rows_pay(P, half, bands[0].gen != 0))
+  if (cfg.rows && rows_pay(P, half, bands[0].gen))
     return launch_force_rows(P, half, bands[0].gen, fuse, s);
   for (int k = 0; k < nb; ++k) {
     const ForceBand &b = bands[k];

@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <iterator>
 
 #include "dpd_device.cuh"
 #include "force_direct.cuh"
@@ -48,13 +49,8 @@ constexpr int kRowsQueue = 1728, kRowsQueueDense = 2880, kRowsQueueDenseHalf = 1
 constexpr int kRowsBlocksFull = 4, kRowsBlocksHalf = 6;
 constexpr unsigned kAll = 0xffffffffu;
 
-// Which boxes (rows_pay).
-constexpr int kRowsMaxHalf = 262144;
-constexpr int kRowsMaxFull = 65536, kRowsMaxFullDense = 106496;  // dense: above 5 per cell
-constexpr int kRowsMaxFullGeneral = 90112, kRowsMaxFullGeneralDense = 139264;
-constexpr int kRowsMaxPerCell = 12;
-bool slots_per_cell_at_most(const Packed &P, int n) {
-  return (long long)P.ntot * kSlicesX <= (long long)n * P.ncell;
+bool slots_per_cell_at_most(const Packed &P, double n) {
+  return (double)P.ntot * kSlicesX <= n * P.ncell;
 }
 
 template <bool HALF, bool DENSE>
@@ -453,27 +449,39 @@ cudaError_t prepare_one() {
 
 }  // namespace
 
-// The row-parallel kernels win while the direct kernels leave the GPU waiting.
-// A step, direct against row-parallel (us):
-//   full  N = 40,960 (rho 10) 78.3 / 47.0; 65,856 (rho 3) 40.5 / 38.3; 81,000 (rho 3)
-//         43.0 / 44.1; 105,456 (rho 6) 73.0 / 65.5; 106,480 (rho 10) 103.9 / 98.3;
-//         279,936 (rho 6) 137.6 / 146.2
-//   half  N = 40,960 (rho 10) 42.5 / 28.4; 192,000 (rho 3) 46.6 / 41.3; 255,552 (rho 3)
-//         52.6 / 51.2; 331,776 (rho 3) 62.0 / 63.9; 552,960 (rho 5) 117.1 / 120.9
-// and the general kernels (Gaussian noise; several species)
-//   full  N = 65,856 (rho 3) 46.1 / 38.9; 42.6 / 38.5, 98,304 (rho 3) 55.2 / 50.2; 49.1 /
-//         49.8, 116,346 (rho 3, uneven edges) 57.5 / 63.9, 138,240 (rho 10) 167.6 / 128.0;
-//         140.6 / 124.9
-//   half  N = 255,552 (rho 3) 55.5 / 53.1; 54.6 / 52.0, 331,776 (rho 3) 66.4 / 66.5; 64.6 / 65.1.
-// Above about 12 particles per cell the lists overflow too often.
-bool rows_pay(const Packed &P, bool half, bool general) {
-  const bool dense = !slots_per_cell_at_most(P, 5);
-  int most = kRowsMaxHalf;
-  if (!half && general)
-    most = dense ? kRowsMaxFullGeneralDense : kRowsMaxFullGeneral;
-  else if (!half)
-    most = dense ? kRowsMaxFullDense : kRowsMaxFull;
-  return P.nbox == 1 && P.ntot <= most && slots_per_cell_at_most(P, kRowsMaxPerCell);
+// The row-parallel kernels win while the direct kernels leave the GPU waiting: the
+// slots up to which they serve a box, by its slots per cell.  A step, row-parallel
+// over direct, on both sides of each line (percent; rho of the box, thousand slots):
+//   full     rho 1    plain 94 (55), 107 (69); Gauss 98 (59), 104 (69); species 94 (55),
+//                     108 (69)
+//            rho 1.5  96 (59), 105 (70); 92 (59), 101 (70); 97 (59), 106 (70)
+//            rho 2    95 (60), 102 (72); 99 (86), 103 (93); 100 (72), 105 (79)
+//            rho 3    97 (73), 101 (81); 98 (128), 96 (140); 98 (81), 101 (89)
+//            rho 5    98 (110), 104 (135); 85 (149); 92 (122), 98 (135)
+//            rho 6    91 (118), 97 (146); 79 (146); 93 (146)
+//            rho 7.3  98 (101), 106 (114); 86 (144); 99 (114), 100 (144)
+//            rho 8    91 (85), 101 (97); 82 (140); 97 (140)
+//            rho 10   92 (106), 96 (138); 75 (138); 90 (138)
+//   half     rho 1    94 (79), 103 (110); 99 (91), 101 (110); 99 (91), 101 (110)
+//            rho 1.5  100 (128), 104 (156); 97 (128), 101 (156); 99 (128), 103 (156)
+//            rho 2    98 (250), 102 (297); 95 (250), 99 (297); 96 (250), 99 (297)
+//            rho 3    98 (255), 101 (292); 96 (255), 100 (292); 96 (255), 99 (292)
+//            rho 10   92 (244), 97 (298); 91 (244), 95 (298); 90 (244), 94 (298)
+// Where a line lies below the crossing, the boxes in between stay on the direct
+// kernel they had.  Above about 12 slots per cell the lists overflow too often.
+bool rows_pay(const Packed &P, bool half, int gen) {
+  struct Limit {
+    double per_cell;
+    int plain, gauss, other;  // other: several species, or both
+  };
+  static constexpr Limit kFull[] = {{1.75, 57344, 57344, 57344},   {3.5, 65536, 90112, 73728},
+                                    {5.0, 65536, 90112, 90112},    {7.0, 106496, 139264, 139264},
+                                    {9.5, 90112, 139264, 139264},  {12.0, 106496, 139264, 139264}};
+  static constexpr Limit kHalf[] = {{1.75, 90112, 90112, 90112}, {12.0, 262144, 262144, 262144}};
+  const Limit *l = half ? kHalf : kFull, *end = half ? std::end(kHalf) : std::end(kFull);
+  while (l != end && !slots_per_cell_at_most(P, l->per_cell)) ++l;
+  if (P.nbox != 1 || l == end) return false;
+  return P.ntot <= (gen == 0 ? l->plain : gen == kGenGauss ? l->gauss : l->other);
 }
 
 cudaError_t prepare_rows() {

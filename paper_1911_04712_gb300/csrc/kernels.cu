@@ -681,7 +681,7 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
   if (P.ntot <= 0) return cudaSuccess;
   const bool half = cfg.stencil == 1;
   const bool early = cfg.rows && P.ntot <= kEarlySlots &&
-                     rows_pay(P, half, cfg.nbands > 0 && cfg.band[0].gen != 0);
+                     rows_pay(P, half, cfg.nbands > 0 ? cfg.band[0].gen : 0);
   // fused_in: row a1 of this step ran in the previous step's force kernel
   if (!fused_in) launch_integrate(P, move, early, s);
   launch_scan(P, advance, early, s);

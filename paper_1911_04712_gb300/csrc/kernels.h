@@ -145,7 +145,7 @@ cudaError_t prepare_rows();
 // out3: also write the forces to id order (n x 3, full stencil).
 cudaError_t launch_force_rows(const Packed &P, bool half, int gen, bool fuse, cudaStream_t s,
                               float *out3 = nullptr);
-bool rows_pay(const Packed &P, bool half, bool general);  // whether they serve this box
+bool rows_pay(const Packed &P, bool half, int gen);  // whether they serve this box
 // The largest such box whose kernels are launched early (step_begin).
 constexpr int kEarlySlots = 65536;
 

@@ -244,7 +244,7 @@ extern "C" int dpd_forces_noalloc(int64_t n, const float *pos, const float *vel,
 
   k_noalloc_bin<<<kNaBlocks, kNaThreads, 0, s>>>(P, pos, vel, (unsigned long long)step);
   DPD_CUDA_TRY(cudaGetLastError());
-  if (rows_pay(P, false, false)) {
+  if (rows_pay(P, false, 0)) {
     DPD_CUDA_TRY(launch_force_rows(P, false, 0, false, s, force));
   } else {
     DPD_CUDA_TRY(launch_force(P, StepConfig{}, s));
