@@ -93,14 +93,24 @@ def force_flops_per_particle(rho: float) -> float:
 # Algorithmic HBM bytes per particle-step of the streaming stages.  The
 # full stencil orders each cell by previous slot (key pass + ranked
 # reorder); the half stencil has no key pass and its reorder places by
-# arrival rank and also zeroes the force it accumulates into.
+# arrival rank and also zeroes the force it accumulates into.  Half-stencil
+# sets of more than EXCHANGE_SLOTS particles run pairs of steps that exchange
+# two pairs of arrays: the first kernel kicks and counts and zeroes the force
+# in place, the reorder drifts again.
+EXCHANGE_SLOTS = 65536
 STAGE_BYTES = {
     "full": {"integrate_bin": 48 + 32 + 8,   # read x, v, f; write x', v', cell, arrival rank
              "bin_keys": 8 + 4,              # read cell, rank; write key
              "bin_scatter": 8 + 32 + 32},    # read cell, start, x', v'; write x, v
     "half": {"integrate_bin": 48 + 32 + 8,
              "bin_scatter": 12 + 32 + 48},   # read cell, rank, start, x', v'; write x, v, f = 0
+    "half_exchange": {"integrate_bin": 48 + 32 + 4,  # read x, v, f; write v', f = 0, arrival rank
+                      "bin_scatter": 36 + 32},       # read x, v', rank; write x', v'
 }
+
+
+def stage_bytes(stencil: str, n: int) -> dict:
+    return STAGE_BYTES["half_exchange" if stencil == "half" and n > EXCHANGE_SLOTS else stencil]
 
 
 # DRAM traffic of the force kernel per launch and its L1 data-pipe
@@ -539,7 +549,7 @@ def run_native(args):
     barrier()
     ms = e0.elapsed_time(e1)
     # ---- per-stage events (same workload, same stream) for the roofline
-    stage_ms = box.profile(args.steps)
+    stage_ms = box.profile(args.steps + args.steps % 2)  # exchanging steps come in pairs
     clk = clocks.stop() if clocks else None
     if clk:
         clk["window"] = "sampled every 200 ms from before a 1 s untimed load through the timed region and the per-stage profile"
@@ -575,8 +585,8 @@ def run_native(args):
     stages = {}
     for name, t in zip(dpd.STAGE_NAMES, stage_ms):
         d = {"ms": round(t, 5), "share": round(t / sum(stage_ms), 4)}
-        if name in STAGE_BYTES[args.stencil]:
-            gbs = STAGE_BYTES[args.stencil][name] * n / (t / 1000.0) / 1e9
+        if name in stage_bytes(args.stencil, n):
+            gbs = stage_bytes(args.stencil, n)[name] * n / (t / 1000.0) / 1e9
             d.update({"GB/s": round(gbs, 1), "hbm_frac": round(gbs / hbm_peak, 3)})
         stages[name] = d
 

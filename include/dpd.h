@@ -233,7 +233,11 @@ DPD_API int64_t dpd_num_particles(const dpd_ctx *ctx);
 /* Advance nsteps steps like dpd_step, launching each step's kernels directly
  * (no graph) with CUDA events recorded on the context's stream between the
  * stages, synchronising after every step.  stage_ms[DPD_NUM_STAGES] receives
- * the mean device milliseconds of each stage. */
+ * the mean device milliseconds of each stage.  The kernels are those of
+ * dpd_step, but for what its steps share or overlap: no fused integrate
+ * (DPD_PARAM_FUSE), no kernel launched before the previous one has drained.
+ * Half-stencil sets above 65,536 slots move their state in pairs of steps; an
+ * odd last step takes the plain kernels, as in dpd_step. */
 DPD_API int dpd_profile_steps(dpd_ctx *ctx, int64_t nsteps, double *stage_ms);
 
 /* ---------------------------------------------------------------- debug */

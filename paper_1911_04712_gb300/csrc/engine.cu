@@ -795,10 +795,11 @@ int Engine::profile(int64_t nsteps, double *stage_ms) {
   if (nsteps <= 0 || ntot_ == 0) return step(nsteps);
   cudaEvent_t ev[kNumStages + 1] = {};
   for (auto &e : ev) DPD_CUDA_TRY(cudaEventCreate(&e));
-  const Packed P = packed();
+  Packed P = packed();
+  const bool swap = swap_pays(P, cfg_);
   int rc = DPD_OK;
   for (int64_t s = 0; s < nsteps && rc == DPD_OK; ++s) {
-    cudaError_t e = launch_step_timed(P, cfg_, stream_, ev);
+    cudaError_t e = launch_step_timed(P, cfg_, swap && (s | 1) < nsteps, stream_, ev);
     if (e == cudaSuccess) e = cudaEventSynchronize(ev[kNumStages]);
     if (e != cudaSuccess) {
       rc = set_error(DPD_ERR_CUDA, "profiled step: %s", cudaGetErrorString(e));

@@ -696,37 +696,52 @@ bool swap_pays(const Packed &P, const StepConfig &cfg) {
   return cfg.stencil == 1 && P.ntot > kSwapSlots;
 }
 
-cudaError_t launch_step_swapped(Packed &P, const StepConfig &cfg, cudaStream_t s) {
-  if (P.ntot <= 0) return cudaSuccess;
+static void launch_kick(const Packed &P, cudaStream_t s) {
   const int gb = blocks_for(P.ntot, kBinThreads);
   if (P.nbox == 1)
     k_kick_bin<true><<<gb, kBinThreads, 0, s>>>(P);
   else
     k_kick_bin<false><<<gb, kBinThreads, 0, s>>>(P);
-  launch_scan(P, true, false, s);
+}
+
+static void launch_drift(Packed &P, cudaStream_t s) {
+  const int gb = blocks_for(P.ntot, kBinThreads);
   if (P.nbox == 1)
     k_drift_scatter<true><<<gb, kBinThreads, 0, s>>>(P);
   else
     k_drift_scatter<false><<<gb, kBinThreads, 0, s>>>(P);
   std::swap(P.pos, P.pos2);
   std::swap(P.vel, P.vel2);
+}
+
+cudaError_t launch_step_swapped(Packed &P, const StepConfig &cfg, cudaStream_t s) {
+  if (P.ntot <= 0) return cudaSuccess;
+  launch_kick(P, s);
+  launch_scan(P, true, false, s);
+  launch_drift(P, s);
   cudaError_t e = cudaGetLastError();
   return e != cudaSuccess ? e : launch_force(P, cfg, s);
 }
 
-cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,
+cudaError_t launch_step_timed(Packed &P, const StepConfig &cfg, bool swap, cudaStream_t s,
                               cudaEvent_t *ev) {
   if (P.ntot <= 0) return cudaSuccess;
   const bool half = cfg.stencil == 1;
   cudaError_t e;
   if ((e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  launch_integrate(P, true, false, s);
+  if (swap)
+    launch_kick(P, s);
+  else
+    launch_integrate(P, true, false, s);
   if ((e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
   launch_scan(P, true, false, s);
   if ((e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
   if (!half) launch_keys(P, false, s);
   if ((e = cudaEventRecord(ev[3], s)) != cudaSuccess) return e;
-  launch_scatter(P, half, false, s);
+  if (swap)
+    launch_drift(P, s);
+  else
+    launch_scatter(P, half, false, s);
   if ((e = cudaEventRecord(ev[4], s)) != cudaSuccess) return e;
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_force(P, cfg, s)) != cudaSuccess) return e;

@@ -381,9 +381,6 @@ cudaError_t launch_load(const Packed &P, int box_slot0, int n, const float *pos3
 cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConfig &cfg,
                         cudaStream_t s, bool fused_in = false, bool fuse_out = false);
 
-// One step with events recorded around its stages: ev[0] before the
-// integrate/count kernel, then after it, after the scan, after the key pass,
-// after the reorder and after the force kernel (6 events).
 // A half-stencil step that moves less (k_kick_bin): the state goes from pos and
 // vel to pos2 and vel2, which are exchanged in P.  Steps come in pairs, so that
 // a call leaves the state where it found it.  A step of an L = 128 box went from
@@ -394,7 +391,10 @@ cudaError_t launch_step(const Packed &P, bool move, bool advance, const StepConf
 cudaError_t launch_step_swapped(Packed &P, const StepConfig &cfg, cudaStream_t s);
 bool swap_pays(const Packed &P, const StepConfig &cfg);
 constexpr int kSwapSlots = 65536;
-cudaError_t launch_step_timed(const Packed &P, const StepConfig &cfg, cudaStream_t s,
+// One step (swap: one that exchanges the arrays) with events recorded around its
+// stages: ev[0] before the integrate/count kernel, then after it, after the scan,
+// after the key pass, after the reorder and after the force kernel (6 events).
+cudaError_t launch_step_timed(Packed &P, const StepConfig &cfg, bool swap, cudaStream_t s,
                               cudaEvent_t *ev);
 constexpr int kNumStages = 5;
 constexpr int kKernelsPerStep = 6;
