@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(NT)
   const bool real = p < B.pbase + B.np;  // lanes past the box's end are dead
   const BoxState S = P.st[G.box[lo]];
   const bool alive = real && S.adv;
-  force_direct<true, NT, CAP, false, false, true>(P, B, S, p, alive, smem_list + threadIdx.x,
+  force_direct<true, NT, CAP, false, 0, true>(P, B, S, p, alive, smem_list + threadIdx.x,
                                                   nullptr, smem_own + (threadIdx.x >> 5) * 64,
                                                   false, false, real);
 }

@@ -136,7 +136,8 @@ inline bool cooperative_variant(int v, bool general, bool half) {
 }
 size_t tile_smem_bytes(int stage_cap);
 // fuse: full stencil only; the kernel also performs the next step's row a1
-// (integrate_one) for every slot and stores no force.
+// (integrate_one) for every slot, and stores the forces of boxes that stop after
+// this step, and under sampling (Packed::keep_frc) all of them.
 cudaError_t launch_force(const Packed &P, const StepConfig &cfg, cudaStream_t s,
                          bool fuse = false);
 

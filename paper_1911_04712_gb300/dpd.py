@@ -425,8 +425,9 @@ _Box3 = ctypes.c_double * 3
 
 
 def _forces_noalloc(torch, dev, n, pos, vel, L, a, gamma, kT, rc, dt, seed, step, out, stream):
-    # Small calls are host-bound (the two launches take about 15 us on the
-    # GPU), so inputs that need no conversion are passed as they are.
+    # Small calls are host-bound (the two kernels take 18 us for 1,536
+    # particles, a call 21), so inputs that need no conversion are passed as
+    # they are.
     def vec3(x):
         if x.dtype != torch.float32 or not x.is_contiguous():
             x = x.detach().to(torch.float32).contiguous()
