@@ -93,14 +93,16 @@ def test_packed_boxes_some_stopped(mods, nsteps):
     ref.close()
 
 
-def test_sampled_half_stencil_set(mods):
-    """A served set above 65,536 slots, sampled at either step of a pair."""
+@pytest.mark.parametrize("steps,every,chunk,samples", [
+    (40, 5, 33, 4),    # a graph of 32 steps: samples behind either step of a pair
+    (20, 11, 20, 1)])  # direct launches: behind step 11, the first of its pair
+def test_sampled_half_stencil_set(mods, steps, every, chunk, samples):
+    """A served set above 65,536 slots, sampled between its exchanging steps."""
     import paper_1911_04712_gb300.serve as S
     D, _ = mods
-    steps, every = 40, 5
     sizes = [(28.2, 66000), (11.0, 4097)]
     states = [uniform_box_state(L, n=n, seed=n) for L, n in sizes]
-    q = S.Queue(1 << 30, chunk_steps=33, sample_every=every, nbins=4, stencil=1)
+    q = S.Queue(1 << 30, chunk_steps=chunk, sample_every=every, nbins=4, stencil=1)
     tk = [q.submit_state(S.make_request(L, n=n, seed=n, steps=steps), x, v)
           for (L, n), (x, v) in zip(sizes, states)]
     q.wait_all(300)
@@ -117,7 +119,7 @@ def test_sampled_half_stencil_set(mods):
                 kT.append(st["kT"])
                 pr.append(st["pressure"])
         box.close()
-        assert g["samples"] == len(kT) == 4
+        assert g["samples"] == len(kT) == samples
         # 40 steps of sums in another order: velocities 1e-4 apart at random, which a
         # mean over 4,000 particles takes to 3e-6
         assert g["kT_mean"] == pytest.approx(np.mean(kT), rel=3e-5)
